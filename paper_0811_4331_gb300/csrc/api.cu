@@ -654,12 +654,12 @@ int vcycle(mg_handle* h, int l, const void* r, void* e, int nrhs) {
   if (xmma) {
     DevBuf scratch;
     const size_t need = (size_t)std::max(fbytes, cbytes);
-    rvar = tuned(h, tkey("restrict_mma", {prec, pc, a.nv, a.bsites, a.Vc, nrhs}), transfer_mma_variants(nrhs),
+    rvar = tuned(h, tkey("restrict_mma", {prec, pc, a.nv, a.bsites, a.Vc, nrhs}), transfer_mma_variants(g, nrhs, false),
                  [&](int v) {
                    if (!scratch.p && !scratch.ensure(need)) return -1;
                    return launch_restrict(prec, prec, pc, g, a.P[prec].p, res, scratch.p, nrhs, h->st, v);
                  });
-    pvar = tuned(h, tkey("prolong_mma", {prec, pc, a.nv, a.bsites, a.Vc, nrhs}), transfer_mma_variants(nrhs),
+    pvar = tuned(h, tkey("prolong_mma", {prec, pc, a.nv, a.bsites, a.Vc, nrhs}), transfer_mma_variants(g, nrhs, true),
                  [&](int v) {
                    if (!scratch.p && !scratch.ensure(need)) return -1;
                    return launch_prolong(pc, prec, prec, g, a.P[prec].p, rc, scratch.p, nrhs, h->st, v);
