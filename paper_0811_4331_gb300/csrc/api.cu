@@ -82,7 +82,7 @@ inline size_t slot_gcr_pre() { return slot_inner(MG_MAX_LEVELS); }  // <w|r>, ||
 inline size_t slot_total() { return slot_gcr_pre() + 4 * kMaxRhs; }
 const int kInnerBasis = 8;
 
-enum { WV_E, WV_RES, WV_P, WV_XC, WV_AXC, WV_RC, WV_EC, WV_T, WV_DT, WV_IN, WV_A, WV_B, WV_KW, WV_KZ, WV_PR, WV_PE, WV_EOA, WV_EOB, WV_EOC, WV_COUNT };
+enum { WV_E, WV_RES, WV_P, WV_XC, WV_AXC, WV_RC, WV_EC, WV_T, WV_DT, WV_IN, WV_A, WV_B, WV_KW, WV_KZ, WV_PR, WV_PE, WV_ROWS, WV_EOA, WV_EOB, WV_EOC, WV_COUNT };
 
 int prec_of(const mg_handle* h, int l) {
   if (!h->p.mixed) return MG_F64;
@@ -296,14 +296,24 @@ int op_apply(mg_handle* h, int l, int prec, const void* in, void* out, const voi
     const double* mmshift = h->mm_active ? h->mm_shift.as<double>() : nullptr;
     // tensor cores: out = a_ A in + c_ y, then the dots in a separate deterministic pass
     const double vb = (double)a.n() * bytes_of(prec);
+    void* rows = nullptr;  // the vectors' BF16 rows
+    if (const size_t rb = coarse_mma_scratch_bytes(a.ncomp, a.V, nrhs)) {
+      rows = work(h, l, prec, WV_ROWS, nrhs, (int)((rb + (size_t)vb * nrhs - 1) / ((size_t)vb * nrhs)));
+      if (!rows) {
+        set_error("no work buffer for the coarse stencil's rows");
+        return MG_ENOMEM;
+      }
+    }
     {
       DevBuf scratch;
       const int var = tuned(h, tkey("coarse_mma", {prec, a.ncomp, a.V, nrhs}), coarse_mma_variants(nrhs), [&](int v) {
         if (!scratch.p && !scratch.ensure((size_t)vb * nrhs)) return -1;
-        return launch_coarse_mma(prec, a.cop_mma.p, in, scratch.p, y, a.L, a.ncomp, nrhs, a_, c_, h->st, v, mmshift);
+        return launch_coarse_mma(prec, a.cop_mma.p, in, scratch.p, y, a.L, a.ncomp, nrhs, a_, c_, h->st, v, mmshift,
+                                 rows);
       });
       Prof pf(h, MG_K_COARSE, MG_BF16, (double)mma_pack_bytes(a.ncomp, a.V) + nrhs * vb * (2 + (y != nullptr)));
-      LK(launch_coarse_mma(prec, a.cop_mma.p, in, out, y, a.L, a.ncomp, nrhs, a_, c_, h->st, var, mmshift));
+      if (rows) count_launches(1);
+      LK(launch_coarse_mma(prec, a.cop_mma.p, in, out, y, a.L, a.ncomp, nrhs, a_, c_, h->st, var, mmshift, rows));
     }
     if (z) {
       Prof pf(h, MG_K_VECTOR, prec, nrhs * vb * (z == out ? 1 : 2));

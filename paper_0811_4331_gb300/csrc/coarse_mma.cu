@@ -11,8 +11,9 @@
 // C_re Y_im into the imaginary tile; -C_im is C_im with the sign bits
 // flipped).  The operator is stored at setup in MMA fragment order,
 // [B][d][tile][kstep][re|im][lane][8 x bf16], so a warp reads 512 contiguous
-// bytes per fragment; the right-hand sides of the 9 neighbours are staged in
-// shared memory as BF16, [d][r][re..., im...].  n is padded to a multiple of
+// bytes per fragment; the right-hand sides are first rounded to BF16 rows
+// [site][r][re..., im...] and those of the 9 neighbours staged in shared
+// memory.  n is padded to a multiple of
 // 16 and R to a multiple of 8 with zeros.
 #include <cuda_bf16.h>
 
@@ -91,82 +92,98 @@ __device__ __forceinline__ void mma_bf16(float (&d)[4], const uint32_t (&a)[4], 
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-template <typename S, int NT8>
-__global__ void coarse_mma_kernel(const uint4* Cf, const S* in, S* out, const S* y2, int L0, int L1, int L2, int L3,
-                                  int n, int npad, int R, float a, float c, const double* shift) {
+// Bytes from one (site, right-hand side) row of BF16 planes (re then im, npad
+// each) to the next: an odd number of 16-byte units, so that eight rows of an
+// ldmatrix fall on distinct banks, in global memory as in shared.
+__host__ __device__ constexpr int row_pitch(int npad) { return 4 * npad + 16; }
+
+// Component-major vectors [R][n][V] -> rows [V][R][re npad | im npad] of BF16.
+// A site's vector is strided by V in memory; gathering it in every CTA that
+// needs it (nine of them) moved each 32-byte sector for 8 bytes, nine times:
+// here each value is read once, coalesced, and the stencil reads whole rows.
+// CTA = 32 sites of one right-hand side, transposed through shared memory.
+template <typename S>
+__global__ void __launch_bounds__(256) coarse_rows_kernel(const S* in, unsigned char* rows, int n, int npad, int V, int R) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __nv_bfloat16* Ys = (__nv_bfloat16*)smem_raw;  // [9][Rpad][2 npad]
-  const int L[4] = {L0, L1, L2, L3};
-  const int V = L0 * L1 * L2 * L3;
-  const int B = blockIdx.x;
-  const int r0 = blockIdx.y * NT8 * 8;  // first right-hand side of this CTA (launch-shape split)
-  const int Rpad = NT8 * 8;
-  const int T = npad / 16;
-  const int KW = 2 * npad;  // one neighbour's row of Ys: re then im
-  int cB[4];
-  site_coords(B, L, cB);
-  // stage the 9 neighbours' right-hand sides as BF16
-  for (int e = threadIdx.x; e < 9 * Rpad * npad; e += blockDim.x) {
-    const int j = e % npad, r = (e / npad) % Rpad, d = e / (npad * Rpad);
-    float re = 0.f, im = 0.f;
-    if (j < n && r0 + r < R) {
-      const cx<float> v = ldc<float>(in, ((size_t)(r0 + r) * n + j) * V + neighbor(cB, L, d));
-      re = v.re;
-      im = v.im;
-    }
-    Ys[((size_t)d * Rpad + r) * KW + j] = __float2bfloat16_rn(re);
-    Ys[((size_t)d * Rpad + r) * KW + npad + j] = __float2bfloat16_rn(im);
+  const int r = blockIdx.y, B0 = blockIdx.x * 32, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int pitch = 4 * npad + 4;  // one bank further per site
+  const S* v = in + (size_t)r * n * V;
+  for (int j = warp; j < npad; j += 8) {
+    cx<float> x = zero<float>();
+    if (j < n && B0 + lane < V) x = ldc<float>(v, (size_t)j * V + B0 + lane);
+    __nv_bfloat16* d = (__nv_bfloat16*)(smem_raw + lane * pitch);
+    d[j] = __float2bfloat16_rn(x.re);
+    d[npad + j] = __float2bfloat16_rn(x.im);
   }
   __syncthreads();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int t = warp;  // row-tile pair owned by this warp
-  if (t >= T) return;
-  const int gid = lane >> 2, tig = lane & 3;
-  float accr[NT8][4], acci[NT8][4];
+  const int words = npad;  // 4-byte words of a row
+  const int ns = min(32, V - B0);
+  for (int b = warp; b < ns; b += 8) {
+    uint32_t* o = (uint32_t*)(rows + ((size_t)(B0 + b) * R + r) * row_pitch(npad));
+    for (int w = lane; w < words; w += 32) o[w] = *(const uint32_t*)(smem_raw + b * pitch + 4 * w);
+  }
+}
+
+// Direct form, for a few right-hand sides (it gathers the nine neighbours'
+// vectors itself: no rows, no second launch) and for stencils whose directions
+// do not fit the ring of the streaming form below.  CTA = one coarse site and
+// NT8 tiles of 8 right-hand sides; warp = row tile t; kAhead operator
+// fragments in flight per warp (two, three, five and nine measured: three).
+constexpr int kAhead = 3;
+// Threads a CTA may have at NT8 (32 T of the launches that fit shared memory): bounds the registers.
+constexpr int mma_threads(int NT8) { return NT8 == 1 ? 1024 : (NT8 == 2 ? 704 : 448); }
+
+// One kstep of a warp's row tile: 16 x 16 of the operator (re, im fragments)
+// times the staged rows at `ya` (this lane's ldmatrix row; matrices re 0-7,
+// re 8-15, im 0-7, im 8-15).
+template <int NT8>
+__device__ __forceinline__ void mma_kstep(float (&accr)[NT8][4], float (&acci)[NT8][4], const uint4& fr, const uint4& fi,
+                                          unsigned ya, int pitch) {
+  const uint32_t Ar[4] = {fr.x, fr.y, fr.z, fr.w};
+  const uint32_t Ai[4] = {fi.x, fi.y, fi.z, fi.w};
+  const uint32_t An[4] = {fi.x ^ 0x80008000u, fi.y ^ 0x80008000u, fi.z ^ 0x80008000u, fi.w ^ 0x80008000u};
+  // groups of four tiles, each product of the group before the next product: an
+  // accumulator's second MMA would otherwise wait out its first one's latency
+  constexpr int QG = NT8 < 4 ? NT8 : 4;
+#pragma unroll
+  for (int q0 = 0; q0 < NT8; q0 += QG) {
+    uint32_t y[QG][4];  // re 0-7, re 8-15, im 0-7, im 8-15
+#pragma unroll
+    for (int u = 0; u < QG; ++u)
+      if (q0 + u < NT8)
+        asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+                     : "=r"(y[u][0]), "=r"(y[u][1]), "=r"(y[u][2]), "=r"(y[u][3])
+                     : "r"(ya + (q0 + u) * 8 * pitch)
+                     : "memory");
+#pragma unroll
+    for (int u = 0; u < QG; ++u)
+      if (q0 + u < NT8) mma_bf16(accr[q0 + u], Ar, y[u][0], y[u][1]);  // C_re Y_re
+#pragma unroll
+    for (int u = 0; u < QG; ++u)
+      if (q0 + u < NT8) mma_bf16(acci[q0 + u], Ai, y[u][0], y[u][1]);  // C_im Y_re
+#pragma unroll
+    for (int u = 0; u < QG; ++u)
+      if (q0 + u < NT8) mma_bf16(accr[q0 + u], An, y[u][2], y[u][3]);  // -C_im Y_im
+#pragma unroll
+    for (int u = 0; u < QG; ++u)
+      if (q0 + u < NT8) mma_bf16(acci[q0 + u], Ar, y[u][2], y[u][3]);  // C_re Y_im
+  }
+}
+
+template <int NT8>
+__device__ __forceinline__ void mma_zero(float (&accr)[NT8][4], float (&acci)[NT8][4]) {
 #pragma unroll
   for (int q = 0; q < NT8; ++q)
 #pragma unroll
     for (int k = 0; k < 4; ++k) accr[q][k] = acci[q][k] = 0.f;
-  const uint4* Cs = Cf + (size_t)B * 9 * T * T * 2 * 32;
-  // (d, s) steps in order; the operator fragments of the next two steps are
-  // loaded while the current one runs, so three 512-byte loads per warp stay
-  // in flight (the stencil is bound by the latency of these reads otherwise)
-  const int KS = 9 * T;
-  auto frag = [&](int k) { return ((((size_t)(k / T) * T + t) * T + (k % T)) * 2) * 32 + lane; };
-  uint4 f0r = __ldg(Cs + frag(0)), f0i = __ldg(Cs + frag(0) + 32);
-  uint4 f1r = f0r, f1i = f0i;
-  if (KS > 1) {
-    f1r = __ldg(Cs + frag(1));
-    f1i = __ldg(Cs + frag(1) + 32);
-  }
-  for (int k = 0; k < KS; ++k) {
-    const int d = k / T, s = k - d * T;
-    const __nv_bfloat16* Yd = Ys + (size_t)d * Rpad * KW;
-    const uint4 fr = f0r, fi = f0i;
-    f0r = f1r;
-    f0i = f1i;
-    if (k + 2 < KS) {
-      f1r = __ldg(Cs + frag(k + 2));
-      f1i = __ldg(Cs + frag(k + 2) + 32);
-    }
-    {
-      const uint32_t Ar[4] = {fr.x, fr.y, fr.z, fr.w};
-      const uint32_t Ai[4] = {fi.x, fi.y, fi.z, fi.w};
-      const uint32_t An[4] = {fi.x ^ 0x80008000u, fi.y ^ 0x80008000u, fi.z ^ 0x80008000u, fi.w ^ 0x80008000u};
-#pragma unroll
-      for (int q = 0; q < NT8; ++q) {
-        const __nv_bfloat16* col = Yd + (size_t)(q * 8 + gid) * KW;
-        const int k0 = s * 16 + 2 * tig;
-        const uint32_t yr0 = *(const uint32_t*)(col + k0), yr1 = *(const uint32_t*)(col + k0 + 8);
-        const uint32_t yi0 = *(const uint32_t*)(col + npad + k0), yi1 = *(const uint32_t*)(col + npad + k0 + 8);
-        mma_bf16(accr[q], Ar, yr0, yr1);  // C_re Y_re
-        mma_bf16(accr[q], An, yi0, yi1);  // -C_im Y_im
-        mma_bf16(acci[q], Ai, yr0, yr1);  // C_im Y_re
-        mma_bf16(acci[q], Ar, yi0, yi1);  // C_re Y_im
-      }
-    }
-  }
-  // epilogue: rows t*16 + gid (+8), right-hand sides q*8 + 2 tig (+1)
+}
+
+// Rows t*16 + gid (+8), right-hand sides r0 + q*8 + 2 tig (+1) of site B.
+template <typename S, int NT8>
+__device__ __forceinline__ void mma_store(const float (&accr)[NT8][4], const float (&acci)[NT8][4], const S* in, S* out,
+                                          const S* y2, const double* shift, int B, int V, int t, int r0, int n, int R,
+                                          float a, float c) {
+  const int lane = threadIdx.x & 31, gid = lane >> 2, tig = lane & 3;
 #pragma unroll
   for (int q = 0; q < NT8; ++q)
 #pragma unroll
@@ -184,6 +201,227 @@ __global__ void coarse_mma_kernel(const uint4* Cf, const S* in, S* out, const S*
     }
 }
 
+template <typename S, int NT8>
+__global__ void __launch_bounds__(mma_threads(NT8))
+    coarse_mma_kernel(const uint4* Cf, const S* in, S* out, const S* y2, int L0, int L1, int L2, int L3, int n, int npad,
+                      int R, float a, float c, const double* shift) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ int nbs[9];
+  const int V = L0 * L1 * L2 * L3;
+  const int B = blockIdx.x;
+  const int r0 = blockIdx.y * NT8 * 8, Rc = min(R - r0, NT8 * 8);  // this CTA's right-hand sides
+  const int T = npad / 16;
+  const int pitch = row_pitch(npad);
+  const int t = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int KS = 9 * T, dskip = (T - 1) * T * 64;  // from a direction's last kstep to the next direction's first
+  uint4 fr[kAhead], fi[kAhead];
+  int ld_s = 0, ld_k = 0;  // position of the next fragment to load
+  const uint4* cp = Cf + (((size_t)B * 9 * T + t) * T * 2) * 32 + lane;
+  auto load = [&](int u) {
+    if (ld_k < KS) {
+      fr[u] = __ldg(cp);
+      fi[u] = __ldg(cp + 32);
+      cp += 64;
+      ++ld_k;
+      if (++ld_s == T) {
+        ld_s = 0;
+        cp += dskip;
+      }
+    }
+  };
+#pragma unroll
+  for (int u = 0; u < kAhead; ++u) load(u);
+  if (threadIdx.x < 9) {
+    const int L[4] = {L0, L1, L2, L3};
+    int cB[4];
+    site_coords(B, L, cB);
+    nbs[threadIdx.x] = neighbor(cB, L, threadIdx.x);
+  }
+  __syncthreads();
+  for (int row = t; row < 9 * Rc; row += T) {
+    const int d = row / Rc, r = row - d * Rc;
+    __nv_bfloat16* o = (__nv_bfloat16*)(smem_raw + (d * NT8 * 8 + r) * pitch);
+    for (int j = lane; j < npad; j += 32) {
+      cx<float> v = zero<float>();
+      if (j < n) v = ldc<float>(in, ((size_t)(r0 + r) * n + j) * V + nbs[d]);
+      o[j] = __float2bfloat16_rn(v.re);
+      o[npad + j] = __float2bfloat16_rn(v.im);
+    }
+  }
+  __syncthreads();
+  float accr[NT8][4], acci[NT8][4];
+  mma_zero<NT8>(accr, acci);
+  unsigned ya = (unsigned)__cvta_generic_to_shared(smem_raw) + (lane & 7) * pitch + ((lane >> 3) & 1) * 16 +
+                (lane >> 4) * 2 * npad;
+  int s = 0;
+  for (int k = 0; k < KS; k += kAhead) {
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u) {
+      if (k + u >= KS) break;
+      const uint4 Ar = fr[u], Ai = fi[u];
+      load(u);
+      mma_kstep<NT8>(accr, acci, Ar, Ai, ya, pitch);
+      ya += 32;
+      if (++s == T) {
+        s = 0;
+        ya += NT8 * 8 * pitch - 32 * T;
+      }
+    }
+  }
+  mma_store<S, NT8>(accr, acci, in, out, y2, shift, B, V, t, r0, n, R, a, c);
+}
+
+// ------------------------------------------------------------------ streaming form
+// A persistent CTA takes (site, group of right-hand sides) items.  Its last
+// warp's first thread streams each item's nine directions -- 9 KB of operator
+// and 5 KB of a neighbour's rows at n = 48 and 24 right-hand sides -- as two
+// bulk copies into a ring of `ns` stages, on into the next items while the T
+// consumer warps (one row tile each) multiply; full and empty are mbarriers
+// per stage.  Bound by the latency of a site's chain of ksteps and its strided
+// 8-byte stores (a component's sites are contiguous, its CTA has one of them),
+// not yet by the 42 MB of operator that 512 sites read.  Directions and ksteps
+// in the direct form's order: the same bits.
+//
+// 16^3 x 32, level 1 (512 sites, n = 48), rows included: 24 right-hand sides
+// 55 -> 19 us, 12 34 -> 14 us.
+__device__ __forceinline__ void mbar_init(unsigned bar, unsigned count) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive(unsigned bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void mbar_expect(unsigned bar, unsigned bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void bulk_copy(unsigned dst, const void* src, unsigned bytes, unsigned bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+               "l"(src), "r"(bytes), "r"(bar)
+               : "memory");
+}
+// Bounded wait for the phase of the given parity; false when it ran out.
+constexpr int kSpinMax = 1 << 18;
+__device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity) {
+  for (int i = 0; i < kSpinMax; ++i) {
+    unsigned ok;
+    asm volatile(
+        "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    if (ok) return true;
+  }
+  return false;
+}
+
+constexpr int kMaxStages = 8;
+
+template <typename S, int NT8>
+__global__ void __launch_bounds__(224)
+    coarse_stream_kernel(const unsigned char* Cf, const S* in, const unsigned char* rows, S* out, const S* y2, int L0,
+                         int L1, int L2, int L3, int n, int npad, int R, float a, float c, const double* shift,
+                         int splits, int items, int ns) {
+  extern __shared__ __align__(128) unsigned char smem_ring[];
+  __shared__ __align__(8) unsigned long long bars[2 * kMaxStages];  // full, empty
+  const int V = L0 * L1 * L2 * L3;
+  const int T = npad / 16, pitch = row_pitch(npad);
+  const unsigned abytes = T * T * 1024, stage = abytes + NT8 * 8 * pitch;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const unsigned ring = (unsigned)__cvta_generic_to_shared(smem_ring);
+  const unsigned full = (unsigned)__cvta_generic_to_shared(bars), empty = full + 8 * kMaxStages;
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < ns; ++i) {
+      mbar_init(full + 8 * i, 1);
+      mbar_init(empty + 8 * i, T);
+    }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncthreads();
+  int slot = 0;
+  unsigned ph = 0;
+  if (warp == T) {  // producer
+    if (lane != 0) return;
+    const int L[4] = {L0, L1, L2, L3};
+    int issued = 0;
+    bool ok = true;
+    for (int w = blockIdx.x; w < items && ok; w += gridDim.x) {
+      const int B = w / splits, r0 = (w - B * splits) * NT8 * 8, Rc = min(R - r0, NT8 * 8);
+      int cB[4];
+      site_coords(B, L, cB);
+      const unsigned rbytes = Rc * pitch;
+#pragma unroll
+      for (int d = 0; d < 9; ++d) {
+        ok = ok && mbar_wait(empty + 8 * slot, ph ^ 1u);
+        if (!ok) break;
+        const unsigned bar = full + 8 * slot, dst = ring + slot * stage;
+        mbar_expect(bar, abytes + rbytes);
+        bulk_copy(dst, Cf + ((size_t)B * 9 + d) * abytes, abytes, bar);
+        bulk_copy(dst + abytes, rows + ((size_t)neighbor(cB, L, d) * R + r0) * pitch, rbytes, bar);
+        ++issued;
+        if (++slot == ns) {
+          slot = 0;
+          ph ^= 1u;
+        }
+      }
+    }
+    // a ring that stopped: its copies land before the CTA's shared memory goes (the consumers report it)
+    if (!ok)
+      for (int i = 0; i < (issued < ns ? issued : ns); ++i) {
+        slot = slot == 0 ? ns - 1 : slot - 1;
+        if (slot == ns - 1) ph ^= 1u;
+        mbar_wait(full + 8 * slot, ph);
+      }
+    return;
+  }
+  const unsigned ya0 = ring + abytes + (lane & 7) * pitch + ((lane >> 3) & 1) * 16 + (lane >> 4) * 2 * npad;
+  const unsigned char* af0 = smem_ring + (size_t)warp * T * 1024 + lane * 16;
+  bool ok = true;
+  for (int w = blockIdx.x; w < items; w += gridDim.x) {
+    const int B = w / splits, r0 = (w - B * splits) * NT8 * 8;
+    float accr[NT8][4], acci[NT8][4];
+    mma_zero<NT8>(accr, acci);
+    for (int d = 0; d < 9; ++d) {
+      ok = ok && mbar_wait(full + 8 * slot, ph);
+      unsigned ya = ya0 + slot * stage;
+      const unsigned char* af = af0 + (size_t)slot * stage;
+#pragma unroll 3
+      for (int s = 0; s < T; ++s) {
+        const uint4 fr = *(const uint4*)af, fi = *(const uint4*)(af + 512);
+        mma_kstep<NT8>(accr, acci, fr, fi, ya, pitch);
+        af += 1024;
+        ya += 32;
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(empty + 8 * slot);
+      if (++slot == ns) {
+        slot = 0;
+        ph ^= 1u;
+      }
+    }
+    if (!ok) accr[0][0] = accr[0][1] = accr[0][2] = accr[0][3] = __int_as_float(0x7fc00000);  // the solver refuses NaN
+    mma_store<S, NT8>(accr, acci, in, out, y2, shift, B, V, warp, r0, n, R, a, c);
+  }
+}
+
+// The streaming form takes stencils of up to kStreamT row tiles: three stages
+// of any group of right-hand sides then fit one CTA's shared memory.
+constexpr int kStreamT = 6;
+// Stages of the ring: what 48 KB hold, at least three.  More CTAs per SM gain
+// more than deeper rings (512 sites, n = 48, 24 right-hand sides: four CTAs of
+// three stages 13.1 us, two of seven 15.4).
+static int stream_stages(int T, int NT8, size_t* stage) {
+  *stage = (size_t)T * T * 1024 + (size_t)NT8 * 8 * row_pitch(16 * T);
+  const int ns = (int)(48 * 1024 / *stage);
+  return ns < 3 ? 3 : (ns > kMaxStages ? kMaxStages : ns);
+}
+
+// Scratch of launch_coarse_mma for R right-hand sides (0: the direct form runs).
+// Below four the gathers cost less than the extra launch.
+constexpr int kRowsFrom = 4;
+size_t coarse_mma_scratch_bytes(int n, int V, int R) {
+  const int T = (n + 15) / 16;
+  return R < kRowsFrom || T > kStreamT ? 0 : (size_t)V * R * row_pitch(16 * T);
+}
+
 // Launch shapes: variant v splits the right-hand sides over CTAs in groups of
 // kMmaTiles[v] tiles of 8 (each output's arithmetic is the same in every shape).
 static const int kMmaTiles[] = {8, 4, 2, 1, 3, 6};
@@ -197,7 +435,7 @@ int coarse_mma_variants(int R) {
 }
 
 int launch_coarse_mma(int prec, const void* Cf, const void* in, void* out, const void* y2, const int L[4], int n, int R,
-                      double a, double c, cudaStream_t st, int variant, const double* shift) {
+                      double a, double c, cudaStream_t st, int variant, const double* shift, void* scratch) {
   if (prec != 1 && prec != 3) return -1;
   const int npad = (n + 15) / 16 * 16, T = npad / 16;
   const int V = L[0] * L[1] * L[2] * L[3];
@@ -209,15 +447,36 @@ int launch_coarse_mma(int prec, const void* Cf, const void* in, void* out, const
       if (kMmaTiles[v] <= NT8all && ++seen == variant) NT8 = kMmaTiles[v];
   }
   const int splits = (NT8all + NT8 - 1) / NT8;
-  const size_t sm = (size_t)9 * NT8 * 8 * 2 * npad * sizeof(__nv_bfloat16);
-  if (sm > 200 * 1024 || T > 32) return -1;
-#define WMG_MMA(S, K)                                                                                    \
-  {                                                                                                      \
-    auto kern = coarse_mma_kernel<S, K>;                                                                 \
-    if (sm > 48 * 1024) allow_big_smem(kern);                                                            \
-    kern<<<dim3(V, splits), 32 * T, sm, st>>>((const uint4*)Cf, (const S*)in, (S*)out, (const S*)y2, L[0], L[1],    \
-                                              L[2], L[3], n,                                                       \
-                                npad, R, (float)a, (float)c, shift);                                     \
+  const size_t sm = (size_t)9 * NT8 * 8 * row_pitch(npad);
+  if ((size_t)9 * NT8 * 8 * 4 * npad > 200 * 1024 || T > 32) return -1;
+  size_t stage = 0;
+  const int ns = stream_stages(T, NT8, &stage);
+  unsigned char* rows = coarse_mma_scratch_bytes(n, V, R) ? (unsigned char*)scratch : nullptr;
+  if (rows) {
+    const size_t smr = (size_t)32 * (4 * npad + 4);
+    const dim3 g((unsigned)((V + 31) / 32), (unsigned)R);
+    if (prec == 1)
+      coarse_rows_kernel<float2><<<g, 256, smr, st>>>((const float2*)in, rows, n, npad, V, R);
+    else
+      coarse_rows_kernel<__nv_bfloat162><<<g, 256, smr, st>>>((const __nv_bfloat162*)in, rows, n, npad, V, R);
+    if (!launched()) return -1;
+  }
+  const int items = V * splits;
+  const size_t ring = (size_t)ns * stage;
+  int ctas = rows ? (int)(224 * 1024 / (ring + 2048)) : 0;  // that shared memory lets an SM hold
+  ctas = (ctas < 1 ? 1 : (ctas > 8 ? 8 : ctas)) * sm_count();
+  if (ctas > items) ctas = items;
+#define WMG_MMA(S, K)                                                                                       \
+  if (rows) {                                                                                               \
+    auto kern = coarse_stream_kernel<S, K>;                                                                 \
+    allow_big_smem(kern);                                                                                   \
+    kern<<<ctas, 32 * (T + 1), ring, st>>>((const unsigned char*)Cf, (const S*)in, rows, (S*)out, (const S*)y2, L[0], \
+                                           L[1], L[2], L[3], n, npad, R, (float)a, (float)c, shift, splits, items, ns); \
+  } else {                                                                                                  \
+    auto kern = coarse_mma_kernel<S, K>;                                                                    \
+    if (sm > 40 * 1024) allow_big_smem(kern);                                                               \
+    kern<<<dim3(V, splits), 32 * T, sm, st>>>((const uint4*)Cf, (const S*)in, (S*)out, (const S*)y2, L[0], L[1], L[2], \
+                                              L[3], n, npad, R, (float)a, (float)c, shift);                 \
   }
 #define WMG_MMA_R(S)                       \
   switch (NT8) {                           \

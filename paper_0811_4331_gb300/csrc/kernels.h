@@ -194,7 +194,11 @@ int launch_mma_pack(const double2* C, int n, int V, void* out, cudaStream_t st);
 // variant >= 0 picks one of coarse_mma_variants(R) launch shapes (right-hand
 // sides split over CTAs); every shape gives bit-identical results.
 int launch_coarse_mma(int prec, const void* Cf, const void* in, void* out, const void* y2, const int L[4], int n, int R,
-                      double a, double c, cudaStream_t st, int variant = -1, const double* shift = nullptr);
+                      double a, double c, cudaStream_t st, int variant = -1, const double* shift = nullptr,
+                      void* scratch = nullptr);
+// scratch: coarse_mma_scratch_bytes (0 for few right-hand sides); without it every CTA gathers its vectors itself,
+// with the same result.
+size_t coarse_mma_scratch_bytes(int n, int V, int R);
 int coarse_mma_variants(int R);
 
 // Aggregation of level l (fine side) into level l+1 (coarse side).
