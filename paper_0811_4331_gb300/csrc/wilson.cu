@@ -96,7 +96,7 @@ struct HopAcc<double, NR> {
 
 // The two hops of direction MU for NR right-hand sides: each link is loaded
 // (and its third row rebuilt) once and applied to every right-hand side.
-template <int MU, int NR, typename R, typename S, typename G, int NL>
+template <int MU, int NR, bool WIDE, typename R, typename S, typename G, int NL>
 __device__ __forceinline__ void hop_pair(HopAcc<R, NR>& acc, const WilsonArgs<S, G, NL>& A, const S* in, int s,
                                          const int (&c)[4], const int (&stride)[4]) {
   const int L = A.L[MU], st = stride[MU];
@@ -107,28 +107,38 @@ __device__ __forceinline__ void hop_pair(HopAcc<R, NR>& acc, const WilsonArgs<S,
 #pragma unroll
   for (int r = 0; r < NR; ++r) {
     cx<R> psi[12];
-    ld_spinor<R, S>(in + r * A.vstride, A.V, fwd, psi);
+    ld_spinor<R, S, WIDE>(in + r * A.vstride, A.V, fwd, psi);
     acc.template add<MU, true>(r, psi, u);
   }
   load_link<R, G, NL>(u, A.U, MU, A.V, bwd);
 #pragma unroll
   for (int r = 0; r < NR; ++r) {
     cx<R> psi[12];
-    ld_spinor<R, S>(in + r * A.vstride, A.V, bwd, psi);
+    ld_spinor<R, S, WIDE>(in + r * A.vstride, A.V, bwd, psi);
     acc.template add<MU, false>(r, psi, u);
   }
+}
+
+// A chunk by 32-byte loads (WIDE: FP32 on a 32-byte boundary) or 16-byte ones.
+template <bool WIDE, typename R, typename S>
+__device__ __forceinline__ void ld_chunk_w(const S* p, size_t i, cx<R> (&v)[4]) {
+  if constexpr (WIDE)
+    ld_chunk_wide<R>(p, i, v);
+  else
+    ld_chunk<R, S>(p, i, v);
 }
 
 // Own-site part of chunk j of a site's output for one right-hand side
 // (pointers offset to it): out = ca in + cb h + cc y, with the dot partials of
 // the value as stored against z.  y or z may alias out, so they are read
 // through the L2 (coherent with this thread's earlier stores).
-template <typename R, typename S>
+// (z == in, the smoother's case, takes the input value at hand).
+template <typename R, typename S, bool WIDE = false>
 __device__ __forceinline__ void finish_chunk(const cx<R> (&h)[4], int j, const S* in, S* out, const S* y, const S* z,
                                              size_t V, int s, R ca, R cb, R cc, R (&red)[3]) {
   const size_t i0 = (size_t)(((unsigned)j * (unsigned)V + (unsigned)s) << 2);
   cx<R> xin[4], yv[4], v[4];
-  ld_chunk<R, S>(in, i0, xin);
+  ld_chunk_w<WIDE, R, S>(in, i0, xin);
   if (y) ld_chunk_cg<R, S>(y, i0, yv);
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
@@ -138,12 +148,11 @@ __device__ __forceinline__ void finish_chunk(const cx<R> (&h)[4], int j, const S
   st_chunk<S, R>(out, i0, v);
   if (z) {
     // reduce the value as stored, so dots see exactly the vector kept
-    cx<R> zz[4];
-    ld_chunk_cg<R, S>(z, i0, zz);
+    if (z != in) ld_chunk_cg<R, S>(z, i0, xin);
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       const cx<R> vs = as_stored<S>(v[k]);
-      const cx<R> d = cmul_conj(vs, zz[k]);
+      const cx<R> d = cmul_conj(vs, xin[k]);
       red[0] += d.re;
       red[1] += d.im;
       red[2] += norm2(vs);
@@ -151,7 +160,7 @@ __device__ __forceinline__ void finish_chunk(const cx<R> (&h)[4], int j, const S
   }
 }
 
-template <typename R, typename S, typename HA>
+template <typename R, typename S, bool WIDE, typename HA>
 __device__ __forceinline__ void finish_site(const HA& acc, int r, const S* in, S* out, const S* y, const S* z, size_t V,
                                             int s, R ca, R cb, R cc, R (&red)[3]) {
 #pragma unroll
@@ -159,7 +168,7 @@ __device__ __forceinline__ void finish_site(const HA& acc, int r, const S* in, S
     cx<R> h[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) h[k] = acc.get(r, 4 * j + k);
-    finish_chunk<R, S>(h, j, in, out, y, z, V, s, ca, cb, cc, red);
+    finish_chunk<R, S, WIDE>(h, j, in, out, y, z, V, s, ca, cb, cc, red);
   }
 }
 
@@ -167,37 +176,37 @@ __device__ __forceinline__ void finish_site(const HA& acc, int r, const S* in, S
 // output and dot partials are computed with the same operations in the same
 // order for any NT and NR, and the dots of right-hand side r are reduced over
 // the same CTAs of NT sites, so a launch shape never changes a result bit.
-// DOTS: the launch reduces <out|z>, ||out||^2 (then every thread of a CTA
-// takes part in the reduction); without it threads past the lattice leave at
-// once and no reduction code runs.
-template <typename S, typename G, int NL, int NT, int NR, bool DOTS>
+// DOTS: the launch reduces <out|z>, ||out||^2; a CTA then takes several tiles
+// of NT sites, because its reduction ends in a fence and an atomic that all
+// its warps wait for.  Without it a thread takes one site and no reduction
+// code runs.  WIDE (FP32): the spinors' chunks as 32-byte loads.
+template <typename S, typename G, int NL, int NT, int NR, bool DOTS, bool WIDE>
 __device__ __forceinline__ void wilson_body(const WilsonArgs<S, G, NL>& A) {
   typedef typename Store<S>::R R;
   const int V = A.V;
-  const int s = blockIdx.x * NT + threadIdx.x;
   const int rhs0 = blockIdx.y * NR;
   const S* in = A.in + rhs0 * A.vstride;
   R red[NR][3];  // per-thread partial dots in the arithmetic type
 #pragma unroll
   for (int r = 0; r < NR; ++r) red[r][0] = red[r][1] = red[r][2] = (R)0;
-  if (!DOTS && s >= V) return;
-  if (s < V) {
+  for (int s = blockIdx.x * NT + threadIdx.x; s < V; s += gridDim.x * NT) {
     int c[4], stride[4];
     site_coords(s, A.L, c, stride);
     HopAcc<R, NR> acc;
     acc.zero();
-    hop_pair<0, NR>(acc, A, in, s, c, stride);
-    hop_pair<1, NR>(acc, A, in, s, c, stride);
-    hop_pair<2, NR>(acc, A, in, s, c, stride);
-    hop_pair<3, NR>(acc, A, in, s, c, stride);
+    hop_pair<0, NR, WIDE>(acc, A, in, s, c, stride);
+    hop_pair<1, NR, WIDE>(acc, A, in, s, c, stride);
+    hop_pair<2, NR, WIDE>(acc, A, in, s, c, stride);
+    hop_pair<3, NR, WIDE>(acc, A, in, s, c, stride);
     const R cb = (R)A.b, cc = (R)A.c;
 #pragma unroll
     for (int r = 0; r < NR; ++r) {
       const R ca = (R)(A.adiag ? A.a * A.adiag[rhs0 + r] : A.a);
       const size_t ro = (size_t)(rhs0 + r) * A.vstride;
-      finish_site<R, S>(acc, r, A.in + ro, A.out + ro, A.y ? A.y + ro : nullptr, DOTS ? A.z + ro : nullptr,
+      finish_site<R, S, WIDE>(acc, r, A.in + ro, A.out + ro, A.y ? A.y + ro : nullptr, DOTS ? A.z + ro : nullptr,
                         (size_t)V, s, ca, cb, cc, red[r]);
     }
+    if (!DOTS) return;  // one site per thread
   }
   if (DOTS) {
 #pragma unroll
@@ -205,18 +214,23 @@ __device__ __forceinline__ void wilson_body(const WilsonArgs<S, G, NL>& A) {
   }
 }
 
-// The plain single-right-hand-side form (no dots) on 16-bit fields is bound
-// by the FP32 pipes: its register budget is capped so that 512 threads fit
-// on an SM.  The other forms keep the compiler's own choice (with FP32
-// fields more registers keep more loads in flight, which is what that
-// memory-bound form needs).
-template <typename S, typename G, int NL, int NT>
-__global__ void __launch_bounds__(NT, 512 / NT) wilson_plain_kernel(const WilsonArgs<S, G, NL> A) {
-  wilson_body<S, G, NL, NT, 1, false>(A);
+// Threads an SM is to hold, i.e. the register budget (65,536 / threads).
+// Measured (us per launch; "-": the compiler's own choice of 96-102, 180 for
+// two right-hand sides per thread):
+//   FP32 plain, 32^3 x 64: - 168, 512 170, 640 158, 768 162
+//   FP32 plain, 16^3 x 32, 12 right-hand sides: - 115, 640 103 (wide loads included)
+//   16-bit plain: 512 135 (384 152, 640 136, 768 138) at 32^3 x 64
+//   two right-hand sides per thread, FP16, 12: - 105, 384 90.5, 512 90.3 (spills)
+//   fused dots, FP16, 12, in several tiles per CTA: - 134, 512 126, 640 131
+// FP64 is bound by its arithmetic pipe at any of them.
+template <typename S, int NR, bool DOTS>
+__host__ __device__ constexpr int wilson_threads() {
+  return sizeof(S) == 16 ? 256 : (NR == 2 ? 384 : (sizeof(S) == 8 && !DOTS ? 640 : 512));
 }
-template <typename S, typename G, int NL, int NT, int NR, bool DOTS>
-__global__ void __launch_bounds__(NT) wilson_kernel(const WilsonArgs<S, G, NL> A) {
-  wilson_body<S, G, NL, NT, NR, DOTS>(A);
+
+template <typename S, typename G, int NL, int NT, int NR, bool DOTS, bool WIDE>
+__global__ void __launch_bounds__(NT, wilson_threads<S, NR, DOTS>() / NT) wilson_kernel(const WilsonArgs<S, G, NL> A) {
+  wilson_body<S, G, NL, NT, NR, DOTS, WIDE>(A);
 }
 
 // Small lattices (a few thousand sites): one thread per site leaves most of
@@ -333,7 +347,7 @@ constexpr int kSmallSites = 32768;
 // is formed on the fly from r and p with the same operations, and rounded to
 // the storage type the same way, as at their own sites, so every site sees
 // the r' that is stored; each thread stores r' and x at its own site.
-template <typename R, typename S>
+template <typename R, typename S, bool WIDE = false>
 struct ShiftedIn {
   const S* r;
   const S* p;
@@ -341,8 +355,8 @@ struct ShiftedIn {
   cx<R> c;
   __device__ __forceinline__ void operator()(int site, cx<R> (&v)[12]) const {
     cx<R> pv[12];
-    ld_spinor<R, S>(r, V, site, v);
-    ld_spinor<R, S>(p, V, site, pv);
+    ld_spinor<R, S, WIDE>(r, V, site, v);
+    ld_spinor<R, S, WIDE>(p, V, site, pv);
 #pragma unroll
     for (int k = 0; k < 12; ++k) v[k] = as_stored<S>(v[k] - c * pv[k]);
   }
@@ -381,13 +395,13 @@ __device__ __forceinline__ cx<R> fused_coef(const MrFuseArgs& F, int rhs) {
 // Own-site part of chunk j of a fused step for one right-hand side (offset
 // ro): x and r' stored, out = a r' + b h, and the dot partials of out
 // against r'.
-template <typename R, typename S>
-__device__ __forceinline__ void fused_chunk(const MrFuseArgs& F, const ShiftedIn<R, S>& in, S* out, size_t ro, int j,
+template <typename R, typename S, bool WIDE>
+__device__ __forceinline__ void fused_chunk(const MrFuseArgs& F, const ShiftedIn<R, S, WIDE>& in, S* out, size_t ro, int j,
                                             int s, const cx<R> (&h)[4], R ca, R cb, R (&red)[3]) {
   const size_t i0 = (j * in.V + s) << 2;
   cx<R> rv[4], pv[4], uv[4], xv[4], v[4];
-  ld_chunk<R, S>(in.r, i0, rv);
-  ld_chunk<R, S>(in.p, i0, pv);
+  ld_chunk_w<WIDE, R, S>(in.r, i0, rv);
+  ld_chunk_w<WIDE, R, S>(in.p, i0, pv);
   if (F.u) ld_chunk<R, S>((const S*)F.u + ro, i0, uv);
   if (F.xin) ld_chunk<R, S>((const S*)F.xin + ro, i0, xv);
 #pragma unroll
@@ -444,7 +458,60 @@ __global__ void __launch_bounds__(NT) wilson_mr_kernel(const WilsonArgs<S, G, NL
       cx<R> h[4];
 #pragma unroll
       for (int k = 0; k < 4; ++k) h[k] = acc[(4 * j + k) / 3][(4 * j + k) % 3];
-      fused_chunk<R, S>(F, in, A.out + ro, ro, j, s, h, (R)A.a, (R)A.b, red);
+      fused_chunk<R, S, false>(F, in, A.out + ro, ro, j, s, h, (R)A.a, (R)A.b, red);
+    }
+  }
+  grid_reduce<3, NT, R>(red, A.red, rhs);
+}
+
+// FP32 (the mixed setup): packed hops, 32-byte loads (WIDE), several tiles of
+// NT sites per CTA, whose coefficient and reduction then cost once.  Bound by
+// latency at the sizes where it runs.  8^3 x 16, 20 candidates: 37.8 -> 29.2 us
+// a step.  (Forming A r' as p - c A p halves the loads and took 28.5 us, but p's
+// recursion left the null vectors ten times further from 64 bits.)
+template <int MU, typename R, typename S, typename G, int NL, bool WIDE>
+__device__ __forceinline__ void mr_hop_pair(HopAcc<R, 1>& acc, const WilsonArgs<S, G, NL>& A,
+                                            const ShiftedIn<R, S, WIDE>& in, int s, const int (&c)[4],
+                                            const int (&stride)[4]) {
+  const int L = A.L[MU], st = stride[MU];
+  const int fwd = (c[MU] == L - 1) ? s - (L - 1) * st : s + st;
+  const int bwd = (c[MU] == 0) ? s + (L - 1) * st : s - st;
+  Link<R> u;
+  cx<R> psi[12];
+  load_link<R, G, NL>(u, A.U, MU, A.V, s);
+  in(fwd, psi);
+  acc.template add<MU, true>(0, psi, u);
+  load_link<R, G, NL>(u, A.U, MU, A.V, bwd);
+  in(bwd, psi);
+  acc.template add<MU, false>(0, psi, u);
+}
+
+constexpr int kMrThreads = 512;  // per SM (640 spills: 35.9 us)
+template <typename S, typename G, int NL, int NT, bool WIDE>
+__global__ void __launch_bounds__(NT, kMrThreads / NT)
+    wilson_mr_tiles_kernel(const WilsonArgs<S, G, NL> A, const MrFuseArgs F) {
+  typedef typename Store<S>::R R;
+  const int V = A.V;
+  const int rhs = blockIdx.y;
+  const cx<R> cf = fused_coef<R>(F, rhs);
+  const size_t ro = (size_t)rhs * A.vstride;
+  const ShiftedIn<R, S, WIDE> in{A.in + ro, (const S*)F.pprev + ro, (size_t)V, cf};
+  R red[3] = {(R)0, (R)0, (R)0};
+  for (int s = blockIdx.x * NT + threadIdx.x; s < V; s += gridDim.x * NT) {
+    int c[4], stride[4];
+    site_coords(s, A.L, c, stride);
+    HopAcc<R, 1> acc;
+    acc.zero();
+    mr_hop_pair<0, R, S, G, NL, WIDE>(acc, A, in, s, c, stride);
+    mr_hop_pair<1, R, S, G, NL, WIDE>(acc, A, in, s, c, stride);
+    mr_hop_pair<2, R, S, G, NL, WIDE>(acc, A, in, s, c, stride);
+    mr_hop_pair<3, R, S, G, NL, WIDE>(acc, A, in, s, c, stride);
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      cx<R> h[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) h[k] = acc.get(0, 4 * j + k);
+      fused_chunk<R, S, WIDE>(F, in, A.out + ro, ro, j, s, h, (R)A.a, (R)A.b, red);
     }
   }
   grid_reduce<3, NT, R>(red, A.red, rhs);
@@ -468,10 +535,25 @@ __global__ void __launch_bounds__(256) wilson_small_mr_kernel(const WilsonArgs<S
   if (warp < 3 && s < V) {
     cx<R> h[4];
     warp_hop_sum<R>(part, warp, h);
-    fused_chunk<R, S>(F, in, A.out + ro, ro, warp, s, h, (R)A.a, (R)A.b, red);
+    fused_chunk<R, S, false>(F, in, A.out + ro, ro, warp, s, h, (R)A.a, (R)A.b, red);
   }
   grid_reduce<3, 256, R>(red, A.red, rhs);
 }
+
+// Tiles per CTA of a launch with fused dots, of which an SM holds `per_sm` CTAs:
+// CTAs of at most about 16 (FP32) or 4 (16-bit) tiles that fill whole waves, so
+// that few tiles pay for a reduction and none waits for a nearly empty last
+// wave; one tile where 16-bit launches have less than eight waves.  (A function
+// of type and sizes alone: every shape of a launch has the same.)  16^3 x 32, 12 right-hand sides, one tile -> 4 / 8 / 16: FP16 134 ->
+// 125.5 / 134 / 136 us, FP32 181 -> 189 / 161 / 150 us.
+static int dot_tiles(unsigned tiles, int nrhs, int per_sm, size_t elem) {
+  const size_t total = (size_t)tiles * nrhs, slots = (size_t)per_sm * sm_count();
+  size_t waves = total / (slots * (elem == 8 ? 16 : 4));
+  if (elem != 8 && total < slots * 8) return 1;
+  waves = waves < 1 ? 1 : waves;
+  return (int)((total + slots * waves - 1) / (slots * waves));
+}
+
 template <typename S, typename G, int NL>
 static int launch_mr_t(const DslashCall& d, const MrFuseArgs& F, cudaStream_t st) {
   WilsonArgs<S, G, NL> A;
@@ -488,26 +570,38 @@ static int launch_mr_t(const DslashCall& d, const MrFuseArgs& F, cudaStream_t st
   A.vstride = (size_t)12 * A.V;
   A.red = d.red;
   A.adiag = nullptr;
-  if constexpr (NL != 9) {
+  if constexpr (NL == 9) {
+    wilson_mr_kernel<S, G, NL, 128><<<dim3((A.V + 127) / 128, d.nrhs), 128, 0, st>>>(A, F);
+  } else {
     if ((size_t)A.V * d.nrhs <= (size_t)kSmallSites) {  // the same split as the unfused stencil
       wilson_small_mr_kernel<S, G, NL><<<dim3((A.V + 31) / 32, d.nrhs), 256, 0, st>>>(A, F);
       return launch_ok() ? 0 : -1;
     }
+    constexpr int NT = 128;
+    const unsigned tiles = (unsigned)((A.V + NT - 1) / NT);
+    const int k = dot_tiles(tiles, d.nrhs, kMrThreads / NT, sizeof(S));
+    const dim3 grid((tiles + k - 1) / k, d.nrhs);
+    if ((((uintptr_t)d.in | (uintptr_t)F.pprev) & 31u) == 0)
+      wilson_mr_tiles_kernel<S, G, NL, NT, true><<<grid, NT, 0, st>>>(A, F);
+    else
+      wilson_mr_tiles_kernel<S, G, NL, NT, false><<<grid, NT, 0, st>>>(A, F);
   }
-  wilson_mr_kernel<S, G, NL, 128><<<dim3((A.V + 127) / 128, d.nrhs), 128, 0, st>>>(A, F);
   return launch_ok() ? 0 : -1;
 }
 
-template <typename S, typename G, int NL, int NT, int NR>
+template <typename S, typename G, int NL, int NT, int NR, bool WIDE = false>
 static int launch_nt(const WilsonArgs<S, G, NL>& A, int nrhs, cudaStream_t st) {
   dim3 grid((A.V + NT - 1) / NT, nrhs / NR);
   if (A.z) {
-    wilson_kernel<S, G, NL, NT, NR, true><<<grid, NT, 0, st>>>(A);
+    if constexpr (NT == 128) {  // the only CTA size of the dots (kShapesDots)
+      const int k = dot_tiles(grid.x, nrhs, wilson_threads<S, 1, true>() / NT, sizeof(S));
+      grid.x = (grid.x + k - 1) / k;
+      wilson_kernel<S, G, NL, NT, NR, true, WIDE><<<grid, NT, 0, st>>>(A);
+    } else {
+      return -1;
+    }
   } else {
-    if constexpr (NR == 1 && sizeof(S) == 4)
-      wilson_plain_kernel<S, G, NL, NT><<<grid, NT, 0, st>>>(A);
-    else
-      wilson_kernel<S, G, NL, NT, NR, false><<<grid, NT, 0, st>>>(A);
+    wilson_kernel<S, G, NL, NT, NR, false, WIDE><<<grid, NT, 0, st>>>(A);
   }
   return launch_ok() ? 0 : -1;
 }
@@ -556,14 +650,19 @@ static int launch_t(const DslashCall& d, cudaStream_t st) {
     WShape sh = {128, 1};
     if (d.variant >= 0 && d.variant < wilson_variants(1, d.z != nullptr, d.nrhs, A.V))
       sh = d.z ? kShapesDots[d.variant] : kShapesFree[d.variant];
-    if (sh.nr == 2) {
-      if (sh.nt == 64) return launch_nt<S, G, NL, 64, 2>(A, d.nrhs, st);
-      if (sh.nt == 256) return launch_nt<S, G, NL, 256, 2>(A, d.nrhs, st);
-      return launch_nt<S, G, NL, 128, 2>(A, d.nrhs, st);
+    if constexpr (sizeof(S) == 8) {
+      // FP32 fields off a 32-byte boundary: 16-byte loads, the default shape
+      if (((uintptr_t)d.in & 31u) != 0) return launch_nt<S, G, NL, 128, 1>(A, d.nrhs, st);
     }
-    if (sh.nt == 64) return launch_nt<S, G, NL, 64, 1>(A, d.nrhs, st);
-    if (sh.nt == 256) return launch_nt<S, G, NL, 256, 1>(A, d.nrhs, st);
-    return launch_nt<S, G, NL, 128, 1>(A, d.nrhs, st);
+    constexpr bool W = sizeof(S) == 8;
+    if (sh.nr == 2) {
+      if (sh.nt == 64) return launch_nt<S, G, NL, 64, 2, W>(A, d.nrhs, st);
+      if (sh.nt == 256) return launch_nt<S, G, NL, 256, 2, W>(A, d.nrhs, st);
+      return launch_nt<S, G, NL, 128, 2, W>(A, d.nrhs, st);
+    }
+    if (sh.nt == 64) return launch_nt<S, G, NL, 64, 1, W>(A, d.nrhs, st);
+    if (sh.nt == 256) return launch_nt<S, G, NL, 256, 1, W>(A, d.nrhs, st);
+    return launch_nt<S, G, NL, 128, 1, W>(A, d.nrhs, st);
   }
 }
 
@@ -573,10 +672,8 @@ int launch_wilson_mr(const DslashCall& d, const void* pprev, const void* u, cons
   switch (d.prec) {
     case 0: return launch_mr_t<double2, double2, 9>(d, F, st);
     case 1: return launch_mr_t<float2, float2, 6>(d, F, st);
-    case 2: return launch_mr_t<__half2, __half2, 6>(d, F, st);
-    case 3: return launch_mr_t<__nv_bfloat162, __nv_bfloat162, 6>(d, F, st);
   }
-  return -1;
+  return -1;  // the setup relaxes in FP64 or FP32
 }
 
 // CTAs per right-hand side of a launch with fused dots (sizes the reduction partials).
