@@ -59,41 +59,6 @@ __device__ __forceinline__ void site_coords(int s, const int (&L)[4], int (&c)[4
   stride[3] = stride[2] * L[2];
 }
 
-// Hopping term of NR right-hand sides at one site: FP32 arithmetic in paired
-// form (Acc2), FP64 in the scalar form.
-template <typename R, int NR>
-struct HopAcc;
-template <int NR>
-struct HopAcc<float, NR> {
-  Acc2 a[NR];
-  __device__ __forceinline__ void zero() {
-#pragma unroll
-    for (int r = 0; r < NR; ++r) acc2_zero(a[r]);
-  }
-  template <int MU, bool FWD>
-  __device__ __forceinline__ void add(int r, const cx<float> (&psi)[12], const Link<float>& u) {
-    hop_packed<MU, FWD>(a[r], psi, u);
-  }
-  __device__ __forceinline__ cx<float> get(int r, int c) const { return acc2_get(a[r], c); }
-};
-template <int NR>
-struct HopAcc<double, NR> {
-  cx<double> a[NR][4][3];
-  __device__ __forceinline__ void zero() {
-#pragma unroll
-    for (int r = 0; r < NR; ++r)
-#pragma unroll
-      for (int sp = 0; sp < 4; ++sp)
-#pragma unroll
-        for (int k = 0; k < 3; ++k) a[r][sp][k] = wmg::zero<double>();
-  }
-  template <int MU, bool FWD>
-  __device__ __forceinline__ void add(int r, const cx<double> (&psi)[12], const Link<double>& u) {
-    hop_vals<MU, FWD, double>(a[r], psi, u);
-  }
-  __device__ __forceinline__ cx<double> get(int r, int c) const { return a[r][c / 3][c % 3]; }
-};
-
 // The two hops of direction MU for NR right-hand sides: each link is loaded
 // (and its third row rebuilt) once and applied to every right-hand side.
 template <int MU, int NR, bool WIDE, typename R, typename S, typename G, int NL>
@@ -117,15 +82,6 @@ __device__ __forceinline__ void hop_pair(HopAcc<R, NR>& acc, const WilsonArgs<S,
     ld_spinor<R, S, WIDE>(in + r * A.vstride, A.V, bwd, psi);
     acc.template add<MU, false>(r, psi, u);
   }
-}
-
-// A chunk by 32-byte loads (WIDE: FP32 on a 32-byte boundary) or 16-byte ones.
-template <bool WIDE, typename R, typename S>
-__device__ __forceinline__ void ld_chunk_w(const S* p, size_t i, cx<R> (&v)[4]) {
-  if constexpr (WIDE)
-    ld_chunk_wide<R>(p, i, v);
-  else
-    ld_chunk<R, S>(p, i, v);
 }
 
 // Own-site part of chunk j of a site's output for one right-hand side

@@ -57,21 +57,30 @@ __device__ __forceinline__ int eo_site(int h, int p, const int (&L)[4], int (&c)
   return c[0] + L[0] * (c[1] + L[1] * (c[2] + L[2] * c[3]));
 }
 
-template <int MU, typename R, typename S, typename G, int NL>
-__device__ __forceinline__ void eo_hop_pair(cx<R> (&acc)[4][3], const EoArgs<S, G, NL>& A, const S* in, int s, int h,
+// The two hops of direction MU.
+template <int MU, bool WIDE, typename R, typename S, typename G, int NL>
+__device__ __forceinline__ void eo_hop_pair(HopAcc<R, 1>& acc, const EoArgs<S, G, NL>& A, const S* in, int s, int h,
                                             const int (&c)[4], const int (&stride)[4]) {
   const int L = A.L[MU], st = stride[MU];
   const int fwd = (c[MU] == L - 1) ? s - (L - 1) * st : s + st;
   const int bwd = (c[MU] == 0) ? s + (L - 1) * st : s - st;
   Link<R> u;
+  cx<R> psi[12];
   load_link<R, G, NL>(u, A.U, MU, A.V, A.parity * A.Vh + h);  // U_mu(n)
-  hop<MU, true>(acc, in, A.Vh, fwd >> 1, u);
+  ld_spinor<R, S, WIDE>(in, A.Vh, fwd >> 1, psi);
+  acc.template add<MU, true>(0, psi, u);
   load_link<R, G, NL>(u, A.U, MU, A.V, (1 - A.parity) * A.Vh + (bwd >> 1));  // U_mu(n - mu)
-  hop<MU, false>(acc, in, A.Vh, bwd >> 1, u);
+  ld_spinor<R, S, WIDE>(in, A.Vh, bwd >> 1, psi);
+  acc.template add<MU, false>(0, psi, u);
 }
 
-template <typename S, typename G, int NL, int NT>
-__global__ void __launch_bounds__(NT) wilson_eo_kernel(const EoArgs<S, G, NL> A) {
+// One thread per half site and right-hand side, packed hops and the register
+// budget of the full stencil (512 threads per SM; 640 and 768, and two
+// right-hand sides per thread at 384 to 512, are 1-5 % slower).  S (two
+// launches) on 16^3 x 32, 12 right-hand sides: FP16 117 -> 110 us, BF16 118 ->
+// 102, FP32 (32-byte loads) 144 -> 129.
+template <typename S, typename G, int NL, int NT, bool DOTS, bool WIDE>
+__global__ void __launch_bounds__(NT, (sizeof(S) == 16 ? 256 : 512) / NT) wilson_eo_kernel(const EoArgs<S, G, NL> A) {
   typedef typename Store<S>::R R;
   const int h = blockIdx.x * NT + threadIdx.x;
   const int rhs = blockIdx.y;
@@ -81,16 +90,13 @@ __global__ void __launch_bounds__(NT) wilson_eo_kernel(const EoArgs<S, G, NL> A)
     int c[4];
     const int s = eo_site(h, A.parity, A.L, c);
     const int stride[4] = {1, A.L[0], A.L[0] * A.L[1], A.L[0] * A.L[1] * A.L[2]};
-    cx<R> acc[4][3];
-#pragma unroll
-    for (int sp = 0; sp < 4; ++sp)
-#pragma unroll
-      for (int k = 0; k < 3; ++k) acc[sp][k] = zero<R>();
+    HopAcc<R, 1> acc;
+    acc.zero();
     const S* in = A.in + ro;
-    eo_hop_pair<0>(acc, A, in, s, h, c, stride);
-    eo_hop_pair<1>(acc, A, in, s, h, c, stride);
-    eo_hop_pair<2>(acc, A, in, s, h, c, stride);
-    eo_hop_pair<3>(acc, A, in, s, h, c, stride);
+    eo_hop_pair<0, WIDE>(acc, A, in, s, h, c, stride);
+    eo_hop_pair<1, WIDE>(acc, A, in, s, h, c, stride);
+    eo_hop_pair<2, WIDE>(acc, A, in, s, h, c, stride);
+    eo_hop_pair<3, WIDE>(acc, A, in, s, h, c, stride);
     const R ca = (R)A.a, cb = (R)A.b, cc = (R)A.c;
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
@@ -101,13 +107,12 @@ __global__ void __launch_bounds__(NT) wilson_eo_kernel(const EoArgs<S, G, NL> A)
       if (A.y) ld_chunk_cg<R, S>(A.y, i0, yv);
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
-        const int c = 4 * j + k;
-        v[k] = cb * acc[c / 3][c % 3];
+        v[k] = cb * acc.get(0, 4 * j + k);
         if (A.x) v[k] = v[k] + ca * xv[k];
         if (A.y) v[k] = v[k] + cc * yv[k];
       }
       st_chunk<S, R>(A.out, i0, v);
-      if (A.z) {
+      if (DOTS) {
         cx<R> zz[4];
         ld_chunk_cg<R, S>(A.z, i0, zz);
 #pragma unroll
@@ -121,12 +126,22 @@ __global__ void __launch_bounds__(NT) wilson_eo_kernel(const EoArgs<S, G, NL> A)
       }
     }
   }
-  if (A.z) grid_reduce<3, NT, R>(red, A.red, rhs);
+  if (DOTS) grid_reduce<3, NT, R>(red, A.red, rhs);
 }
 
 constexpr int kEoThreads = 128;
 
 int eo_blocks(int V) { return (V / 2 + kEoThreads - 1) / kEoThreads; }
+
+template <typename S, typename G, int NL, bool WIDE>
+static int launch_eo_w(const EoArgs<S, G, NL>& A, int nrhs, cudaStream_t st) {
+  const dim3 grid(eo_blocks(A.V), nrhs);
+  if (A.z)
+    wilson_eo_kernel<S, G, NL, kEoThreads, true, WIDE><<<grid, kEoThreads, 0, st>>>(A);
+  else
+    wilson_eo_kernel<S, G, NL, kEoThreads, false, WIDE><<<grid, kEoThreads, 0, st>>>(A);
+  return launched() ? 0 : -1;
+}
 
 template <typename S, typename G, int NL>
 static int launch_eo_t(const EoCall& d, cudaStream_t st) {
@@ -145,9 +160,10 @@ static int launch_eo_t(const EoCall& d, cudaStream_t st) {
   A.b = d.b;
   A.c = d.c;
   A.red = d.red;
-  dim3 grid(eo_blocks(A.V), d.nrhs);
-  wilson_eo_kernel<S, G, NL, kEoThreads><<<grid, kEoThreads, 0, st>>>(A);
-  return launched() ? 0 : -1;
+  if constexpr (sizeof(S) == 8) {
+    if (((uintptr_t)d.in & 31u) == 0) return launch_eo_w<S, G, NL, true>(A, d.nrhs, st);
+  }
+  return launch_eo_w<S, G, NL, false>(A, d.nrhs, st);
 }
 
 int launch_wilson_eo(const EoCall& d, cudaStream_t st) {

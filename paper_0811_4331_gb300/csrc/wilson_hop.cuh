@@ -144,6 +144,15 @@ __device__ __forceinline__ void st_chunk(S* p, size_t i, const cx<R> (&v)[4]) {
   }
 }
 
+// A chunk by 32-byte loads (WIDE: FP32 on a 32-byte boundary) or 16-byte ones.
+template <bool WIDE, typename R, typename S>
+__device__ __forceinline__ void ld_chunk_w(const S* p, size_t i, cx<R> (&v)[4]) {
+  if constexpr (WIDE)
+    ld_chunk_wide<R>(p, i, v);
+  else
+    ld_chunk<R, S>(p, i, v);
+}
+
 // All 12 components of site s of a level-0 field with V sites (offsets within
 // one field in 32-bit arithmetic: 12 V < 2^32).
 template <typename R, typename S, bool WIDE = false>
@@ -357,5 +366,40 @@ __device__ __forceinline__ void hop_packed(Acc2& A, const cx<float> (&psi)[12], 
     }
   }
 }
+
+// Hopping term of NR right-hand sides at one site: FP32 arithmetic in paired
+// form (Acc2), FP64 in the scalar form.
+template <typename R, int NR>
+struct HopAcc;
+template <int NR>
+struct HopAcc<float, NR> {
+  Acc2 a[NR];
+  __device__ __forceinline__ void zero() {
+#pragma unroll
+    for (int r = 0; r < NR; ++r) acc2_zero(a[r]);
+  }
+  template <int MU, bool FWD>
+  __device__ __forceinline__ void add(int r, const cx<float> (&psi)[12], const Link<float>& u) {
+    hop_packed<MU, FWD>(a[r], psi, u);
+  }
+  __device__ __forceinline__ cx<float> get(int r, int c) const { return acc2_get(a[r], c); }
+};
+template <int NR>
+struct HopAcc<double, NR> {
+  cx<double> a[NR][4][3];
+  __device__ __forceinline__ void zero() {
+#pragma unroll
+    for (int r = 0; r < NR; ++r)
+#pragma unroll
+      for (int sp = 0; sp < 4; ++sp)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) a[r][sp][k] = wmg::zero<double>();
+  }
+  template <int MU, bool FWD>
+  __device__ __forceinline__ void add(int r, const cx<double> (&psi)[12], const Link<double>& u) {
+    hop_vals<MU, FWD, double>(a[r], psi, u);
+  }
+  __device__ __forceinline__ cx<double> get(int r, int c) const { return a[r][c / 3][c % 3]; }
+};
 
 }  // namespace wmg
