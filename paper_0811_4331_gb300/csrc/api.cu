@@ -137,7 +137,9 @@ int ensure_reducer(mg_handle* h, int nrhs) {
   size_t need = (size_t)kMaxVecBlocks * 16 * ((kMaxBasis / 8) * (size_t)nrhs + 1);
   for (auto& lp : h->lev) {
     const Level& a = *lp;
-    size_t b = a.q == 4 ? (size_t)wilson_blocks(a.V) : (size_t)coarse_blocks(a.ncomp, a.V);  // level 0: the stencil
+    // level 0: the stencil
+    size_t b = a.q == 4 ? (size_t)wilson_blocks(a.V)
+                        : (size_t)std::max(coarse_blocks(a.ncomp, a.V, 1), coarse_blocks(a.ncomp, a.V, nrhs));
     need = std::max(need, b * 3 * (size_t)nrhs);
   }
   if (need <= h->red.max_partials && h->red.nslots) return MG_OK;

@@ -11,6 +11,8 @@
 // site of the aggregate in x-fastest order): the restriction of one coarse
 // component is a contiguous dot product and the prolongation of one fine
 // component a contiguous column read.
+#include <algorithm>
+
 #include "common.cuh"
 #include "kernels.h"
 
@@ -34,131 +36,249 @@ struct CoarseArgs {
   const double* shift;  // null, or a diagonal shift per right-hand side
 };
 
-// G lanes cooperate on one output (i, B): lane q of the group sums the
-// (d, j) terms q, q + G, ...; the group then reduces with shuffles.  Small
-// coarse grids use large G so that the launch still covers every SM.
-template <typename S, int NT, int G>
-__global__ void __launch_bounds__(NT) coarse_apply_kernel(const CoarseArgs<S> A) {
+// BV consecutive stored complex elements (16 bytes, or one) as type R.
+template <int BV, typename R, typename S>
+__device__ __forceinline__ void ld_sites(const S* p, cx<R> (&v)[BV]) {
+  if constexpr (BV == 1) {
+    v[0] = ldc<R>(p, 0);
+  } else if constexpr (sizeof(S) == 8) {
+    const float4 q = __ldg(reinterpret_cast<const float4*>(p));
+    v[0] = mk<R>((R)q.x, (R)q.y);
+    v[1] = mk<R>((R)q.z, (R)q.w);
+  } else {
+    const uint4 q = __ldg(reinterpret_cast<const uint4*>(p));
+    const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[k] = ldc<R>(reinterpret_cast<const S*>(&w[k]), 0);
+  }
+}
+
+// CTA = LB x BV consecutive sites, IR rows i and RB right-hand sides; its 256
+// threads are LB groups of BV sites times 256 / LB slices of the 9 n terms
+// (d, j).  A thread reads BV sites of a matrix element as one 16-byte load for
+// each of its IR rows, and the neighbour's component once for all of them;
+// the slices are added by shuffles within a warp and in warp order across the
+// CTA (deterministic).  With one right-hand side the operator's bytes bound it
+// (85 MB on 512 sites, n = 48, FP32), with several in FP64 the FP64 pipe.
+// The operator is read once per RB right-hand sides.
+// 512 sites, n = 48, FP32, one right-hand side: 33 -> 20.7 us, 12: 243 -> 77; 32
+// sites, FP64, one (n = 40): 16.5 -> 12.5 us, 12 (n = 48): 97 -> 66.
+template <typename S, int BV, int IR, int RB, int LB>
+__global__ void __launch_bounds__(256) coarse_apply_kernel(const CoarseArgs<S> A, int nrhs) {
   typedef typename Store<S>::R R;
+  constexpr int SL = 256 / LB, NO = LB * BV * IR;  // slices; outputs per right-hand side
+  __shared__ R part[8 * 2 * NO];  // [warp][re, im][output] of one right-hand side at a time
+  __shared__ int nbs[9][LB * BV];
   const int V = A.V, n = A.n;
-  const int t = blockIdx.x * NT + threadIdx.x;
-  const int o = t / G, q = t % G;  // output index o = i V + B
-  const int rhs = blockIdx.y;
-  const size_t voff = (size_t)rhs * n * V;
-  R red[3] = {(R)0, (R)0, (R)0};
-  const bool live = o < n * V;
-  cx<R> acc = zero<R>();
-  int i = 0, B = 0;
-  if (live) {
-    i = o / V;
-    B = o - i * V;
+  const int nbb = (V + LB * BV - 1) / (LB * BV);
+  const int Bc = (blockIdx.x % nbb) * LB * BV, i0 = (blockIdx.x / nbb) * IR, r0 = blockIdx.y * RB;
+  const int bl = threadIdx.x % LB, sl = threadIdx.x / LB;
+  for (int e = threadIdx.x; e < 9 * LB * BV; e += 256) {
+    const int d = e / (LB * BV), b = e - d * LB * BV;
     int c[4];
-    site_coords(B, A.L, c);
-    const int terms = 9 * n;
-    int d = q / n, j = q - (q / n) * n;
-    int nb = (q < terms) ? neighbor(c, A.L, d) : 0;
-    auto next = [&]() {
-      j += G;
+    site_coords(min(Bc + b, V - 1), A.L, c);
+    nbs[d][b] = neighbor(c, A.L, d);
+  }
+  __syncthreads();
+  cx<R> acc[RB][IR][BV];
+#pragma unroll
+  for (int r = 0; r < RB; ++r)
+#pragma unroll
+    for (int i = 0; i < IR; ++i)
+#pragma unroll
+      for (int v = 0; v < BV; ++v) acc[r][i][v] = zero<R>();
+  const int B0 = Bc + bl * BV;
+  if (B0 < V) {
+    // rows past n and right-hand sides past the last repeat the last one; neither is stored
+    const S* Ci[IR];
+    const S* xr[RB];
+#pragma unroll
+    for (int i = 0; i < IR; ++i) Ci[i] = A.C + (size_t)min(i0 + i, n - 1) * n * V + B0;
+#pragma unroll
+    for (int r = 0; r < RB; ++r) xr[r] = A.in + (size_t)min(r0 + r, nrhs - 1) * n * V;
+    const size_t dstep = (size_t)n * n * V;
+    int d = sl / n, j = sl - d * n;
+    auto term = [&](cx<R> (&cv)[IR][BV], cx<R> (&xv)[RB][BV]) {
+      const size_t o = d * dstep + (size_t)j * V;
+#pragma unroll
+      for (int i = 0; i < IR; ++i) ld_sites<BV, R, S>(Ci[i] + o, cv[i]);
+#pragma unroll
+      for (int r = 0; r < RB; ++r)
+#pragma unroll
+        for (int v = 0; v < BV; ++v) xv[r][v] = ldc<R>(xr[r], (size_t)j * V + nbs[d][bl * BV + v]);
+      j += SL;
       while (j >= n) {
         j -= n;
         ++d;
-        if (d < 9) nb = neighbor(c, A.L, d);
       }
     };
-    int p = q;
-    // four terms' loads in flight per lane (the sum keeps its order)
-    for (; p + 3 * G < terms; p += 4 * G) {
-      cx<R> cv[4], xv[4];
+    auto add = [&](const cx<R> (&cv)[IR][BV], const cx<R> (&xv)[RB][BV]) {
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        cv[u] = ldc<R>(A.C, (((size_t)(d * n + i) * n) + j) * V + B);
-        xv[u] = ldc<R>(A.in, voff + (size_t)j * V + nb);
-        next();
+      for (int r = 0; r < RB; ++r)
+#pragma unroll
+        for (int i = 0; i < IR; ++i)
+#pragma unroll
+          for (int v = 0; v < BV; ++v) acc[r][i][v] = cfma(cv[i][v], xv[r][v], acc[r][i][v]);
+    };
+    constexpr int U = (RB * BV + 2 * IR * BV) * sizeof(R) > 64 ? 2 : 4;  // terms whose loads are in flight together
+    int p = sl;
+    for (; p + (U - 1) * SL < 9 * n; p += U * SL) {
+      cx<R> cv[U][IR][BV], xv[U][RB][BV];
+#pragma unroll
+      for (int u = 0; u < U; ++u) term(cv[u], xv[u]);
+#pragma unroll
+      for (int u = 0; u < U; ++u) add(cv[u], xv[u]);
+    }
+    for (; p < 9 * n; p += SL) {
+      cx<R> cv[IR][BV], xv[RB][BV];
+      term(cv, xv);
+      add(cv, xv);
+    }
+  }
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  R red[RB][3];
+#pragma unroll
+  for (int r = 0; r < RB; ++r) {
+    if (r > 0) __syncthreads();  // the previous right-hand side's sums are read
+#pragma unroll
+    for (int i = 0; i < IR; ++i)
+#pragma unroll
+      for (int v = 0; v < BV; ++v) {
+        cx<R> s = acc[r][i][v];
+#pragma unroll
+        for (int w = LB; w < 32; w <<= 1) {
+          s.re += __shfl_xor_sync(0xffffffffu, s.re, w);
+          s.im += __shfl_xor_sync(0xffffffffu, s.im, w);
+        }
+        if (lane < LB) {
+          R* o = part + warp * 2 * NO + (i * BV + v) * LB + lane;
+          o[0] = s.re;
+          o[NO] = s.im;
+        }
       }
+    __syncthreads();
+    red[r][0] = red[r][1] = red[r][2] = (R)0;
 #pragma unroll
-      for (int u = 0; u < 4; ++u) acc = cfma(cv[u], xv[u], acc);
-    }
-    for (; p < terms; p += G) {
-      acc = cfma(ldc<R>(A.C, (((size_t)(d * n + i) * n) + j) * V + B), ldc<R>(A.in, voff + (size_t)j * V + nb), acc);
-      next();
-    }
-  }
-  if (G > 1) {
+    for (int o = threadIdx.x; o < NO; o += 256) {
+      const int B = Bc + (o % LB) * BV + (o / LB) % BV, i = i0 + o / (LB * BV);
+      if (B >= V || i >= n || r0 + r >= nrhs) continue;
+      cx<R> s = zero<R>();
 #pragma unroll
-    for (int w = G / 2; w > 0; w >>= 1) {
-      acc.re += __shfl_xor_sync(0xffffffffu, acc.re, w);
-      acc.im += __shfl_xor_sync(0xffffffffu, acc.im, w);
+      for (int w = 0; w < 8; ++w) s = s + mk<R>(part[w * 2 * NO + o], part[w * 2 * NO + NO + o]);
+      const size_t oo = ((size_t)(r0 + r) * n + i) * V + B;
+      if (A.shift) s = cfma(mk<R>((R)A.shift[r0 + r], (R)0), ldc<R>(A.in, oo), s);
+      cx<R> v = (R)A.a * s;
+      if (A.y) v = v + (R)A.c * ldc<R>(A.y, oo);
+      stc(A.out, oo, v);
+      if (A.z) {
+        const cx<R> vs = as_stored<S>(v);
+        const cx<R> dd = cmul_conj(vs, ldc<R>(A.z, oo));
+        red[r][0] += dd.re;
+        red[r][1] += dd.im;
+        red[r][2] += norm2(vs);
+      }
     }
   }
-  if (live && q == 0) {
-    const size_t oo = voff + (size_t)i * V + B;
-    if (A.shift) acc = cfma(mk<R>((R)A.shift[rhs], (R)0), ldc<R>(A.in, oo), acc);
-    cx<R> v = (R)A.a * acc;
-    if (A.y) v = v + (R)A.c * ldc<R>(A.y, oo);
-    stc(A.out, oo, v);
-    if (A.z) {
-      const cx<R> vs = as_stored<S>(v);
-      const cx<R> dd = cmul_conj(vs, ldc<R>(A.z, oo));
-      red[0] = dd.re;
-      red[1] = dd.im;
-      red[2] = norm2(vs);
-    }
+  if (A.z) {
+#pragma unroll
+    for (int r = 0; r < RB; ++r)
+      if (r0 + r < nrhs) grid_reduce<3, 256, R>(red[r], A.red, r0 + r);
   }
-  if (A.z) grid_reduce<3, NT, R>(red, A.red, rhs);
 }
 
-// Lanes per output: enough threads for ~64K in flight, at most 32.
-static int coarse_group(int ncomp, int V) {
-  const long outs = (long)ncomp * V;
-  int G = 1;
-  while (G < 32 && outs * G < 65536) G *= 2;
-  return G;
+// Tile of a launch.  Up to kCoarseLarge outputs: 16 site groups and the most
+// rows (4, 2, 1) that leave two CTAs per SM -- rows share the vector's loads,
+// but few CTAs leave the GPU idle (32 sites, n = 48, 12 right-hand sides, FP32:
+// 10.6 us with one row, 16.7 with four; 512 sites: 103 with two, 76 with four;
+// one right-hand side 20.7 with two, 27.8 with one).  FP64 takes one row: it is
+// bound by its arithmetic and wants CTAs, and no lane for a right-hand side that is
+// not there.  Above, 32 site groups, and for one right-hand side rows enough to
+// keep the reduction partials few.
+constexpr long kCoarseLarge = 65536;
+static long coarse_ctas(int n, int V, int lb_bv, int ir) {
+  return (long)((V + lb_bv - 1) / lb_bv) * ((n + ir - 1) / ir);
 }
 
-int launch_coarse_apply(const CoarseCall& k, cudaStream_t st) {
-  constexpr int NT = 128;
-  const int V = k.L[0] * k.L[1] * k.L[2] * k.L[3];
-  const int G = coarse_group(k.ncomp, V);
-  dim3 grid((unsigned)(((long)k.ncomp * V * G + NT - 1) / NT), k.nrhs);
-#define WMG_COARSE_G(S, GG) coarse_apply_kernel<S, NT, GG><<<grid, NT, 0, st>>>(A)
-#define WMG_COARSE(S)                                        \
-  {                                                          \
-    CoarseArgs<S> A;                                         \
-    A.C = (const S*)k.C;                                     \
-    A.in = (const S*)k.in;                                   \
-    A.out = (S*)k.out;                                       \
-    A.y = (const S*)k.y;                                     \
-    A.z = (const S*)k.z;                                     \
-    for (int q = 0; q < 4; ++q) A.L[q] = k.L[q];             \
-    A.V = V;                                                 \
-    A.n = k.ncomp;                                           \
-    A.a = k.a;                                               \
-    A.c = k.c;                                               \
-    A.red = k.red;                                           \
-    A.shift = k.shift;                                       \
-    switch (G) {                                             \
-      case 1: WMG_COARSE_G(S, 1); break;                     \
-      case 2: WMG_COARSE_G(S, 2); break;                     \
-      case 4: WMG_COARSE_G(S, 4); break;                     \
-      case 8: WMG_COARSE_G(S, 8); break;                     \
-      case 16: WMG_COARSE_G(S, 16); break;                   \
-      default: WMG_COARSE_G(S, 32); break;                   \
-    }                                                        \
-  }
-  switch (k.prec) {
-    case 0: WMG_COARSE(double2); break;
-    case 1: WMG_COARSE(float2); break;
-    case 2: WMG_COARSE(__half2); break;
-    case 3: WMG_COARSE(__nv_bfloat162); break;
-    default: return -1;
-  }
-#undef WMG_COARSE
-#undef WMG_COARSE_G
+template <typename S, int BV, int IR, int RB, int LB>
+static int coarse_go(const CoarseArgs<S>& A, int nrhs, cudaStream_t st) {
+  const dim3 grid((unsigned)coarse_ctas(A.n, A.V, LB * BV, IR), (unsigned)((nrhs + RB - 1) / RB));
+  coarse_apply_kernel<S, BV, IR, RB, LB><<<grid, 256, 0, st>>>(A, nrhs);
   return launched() ? 0 : -1;
 }
 
-int coarse_blocks(int ncomp, int V) {
-  return (int)(((long)ncomp * V * coarse_group(ncomp, V) + 127) / 128);
+template <typename S, int BV, int RB>
+static int coarse_launch(const CoarseArgs<S>& A, int nrhs, cudaStream_t st) {
+  constexpr bool f64 = sizeof(S) == 16;
+  if ((long)A.n * A.V >= kCoarseLarge) {
+    if constexpr (RB == 1)
+      return nrhs == 1 ? coarse_go<S, BV, BV == 1 ? 4 : 2, 1, 32>(A, nrhs, st) : coarse_go<S, BV, 1, 1, 32>(A, nrhs, st);
+    else
+      return coarse_go<S, BV, f64 ? 1 : (RB == 4 ? 4 : 2), RB, 32>(A, nrhs, st);
+  }
+  const long gy = (nrhs + RB - 1) / RB, want = 2L * sm_count();
+  if constexpr (!f64) {
+    if constexpr (RB == 4)
+      if (coarse_ctas(A.n, A.V, 16 * BV, 4) * gy >= want) return coarse_go<S, BV, 4, RB, 16>(A, nrhs, st);
+    if (coarse_ctas(A.n, A.V, 16 * BV, 2) * gy >= want) return coarse_go<S, BV, 2, RB, 16>(A, nrhs, st);
+  } else {
+    // half the slices are half the additions that join them
+    if (coarse_ctas(A.n, A.V, 32, 1) * gy >= 2 * want) return coarse_go<S, BV, 1, RB, 32>(A, nrhs, st);
+  }
+  return coarse_go<S, BV, 1, RB, 16>(A, nrhs, st);
+}
+
+template <typename S>
+static int coarse_launch_s(const CoarseCall& k, int V, cudaStream_t st) {
+  CoarseArgs<S> A;
+  A.C = (const S*)k.C;
+  A.in = (const S*)k.in;
+  A.out = (S*)k.out;
+  A.y = (const S*)k.y;
+  A.z = (const S*)k.z;
+  for (int q = 0; q < 4; ++q) A.L[q] = k.L[q];
+  A.V = V;
+  A.n = k.ncomp;
+  A.a = k.a;
+  A.c = k.c;
+  A.red = k.red;
+  A.shift = k.shift;
+  constexpr int BV = (int)(16 / sizeof(S));
+  if constexpr (BV > 1) {
+    if (V % BV != 0)  // a row of sites does not start on 16 bytes
+      return k.nrhs == 1 ? coarse_launch<S, 1, 1>(A, 1, st) : coarse_launch<S, 1, 4>(A, k.nrhs, st);
+  }
+  if (k.nrhs == 1 || (sizeof(S) == 16 && k.nrhs % 2)) return coarse_launch<S, BV, 1>(A, k.nrhs, st);
+  if (k.nrhs == 2 || sizeof(S) == 16) return coarse_launch<S, BV, 2>(A, k.nrhs, st);
+  if constexpr (sizeof(S) < 16) return coarse_launch<S, BV, 4>(A, k.nrhs, st);
+  return -1;
+}
+
+int launch_coarse_apply(const CoarseCall& k, cudaStream_t st) {
+  const int V = k.L[0] * k.L[1] * k.L[2] * k.L[3];
+  switch (k.prec) {
+    case 0: return coarse_launch_s<double2>(k, V, st);
+    case 1: return coarse_launch_s<float2>(k, V, st);
+    case 2: return coarse_launch_s<__half2>(k, V, st);
+    case 3: return coarse_launch_s<__nv_bfloat162>(k, V, st);
+  }
+  return -1;
+}
+
+// CTAs of a launch per right-hand side, at most (sizes the reduction partials;
+// not below the count this function has always given).
+int coarse_blocks(int ncomp, int V, int nrhs) {
+  const long outs = (long)ncomp * V;
+  long G = 1;
+  while (G < 32 && outs * G < 65536) G *= 2;
+  long most = (outs * G + 127) / 128;
+  long c;
+  if (outs < kCoarseLarge)
+    c = coarse_ctas(ncomp, V, 16, 1);
+  else if (nrhs == 1)
+    c = std::max(coarse_ctas(ncomp, V, 32, 4), V % 2 ? 0L : coarse_ctas(ncomp, V, 64, 2));
+  else
+    c = coarse_ctas(ncomp, V, 32, 1);
+  return (int)(c > most ? c : most);
 }
 
 // ------------------------------------------------------------------ aggregates

@@ -118,7 +118,7 @@ extern "C" int mr_apply_noalloc(mg_handle* h, int level, int prec, const void* b
   // carve the fixed scratch: p | partial sums | tickets | result slot
   const size_t n = a.n();
   const size_t partials = mma ? (size_t)red_blocks(n) * 4
-                               : (level == 0 ? (size_t)wilson_blocks(a.V) : (size_t)coarse_blocks(a.ncomp, a.V)) * 3;
+                               : (level == 0 ? (size_t)wilson_blocks(a.V) : (size_t)coarse_blocks(a.ncomp, a.V, 1)) * 3;
   const size_t off_part = align256(n * elem_bytes(prec));
   const size_t off_tick = off_part + align256(partials * sizeof(double));
   const size_t off_slot = off_tick + 256;
