@@ -58,6 +58,7 @@ __device__ __forceinline__ cx<R> mr_alpha(const MrUpdate& m, int rhs) {
 
 template <typename S>
 __global__ void __launch_bounds__(kVecThreads) mr_update_kernel(const MrUpdate m) {
+  chain_begin();
   typedef typename Store<S>::R R;
   const int rhs = blockIdx.y;
   const cx<R> alpha = mr_alpha<R>(m, rhs);
@@ -91,6 +92,7 @@ struct __align__(8) Pair16 {
 
 template <typename S>
 __global__ void __launch_bounds__(kVecThreads) mr_update2_kernel(const MrUpdate m) {
+  chain_begin();
   typedef Pair16<S> P2;
   const int rhs = blockIdx.y;
   const cx<float> alpha = mr_alpha<float>(m, rhs);
@@ -132,19 +134,19 @@ int launch_mr_update(const MrUpdate& m, cudaStream_t st) {
                      al8(m.x_in) && al8(m.u) && al8(m.r_out) && al8(m.r_in) && al8(m.p);
   if (pairs) grid.x = vec_blocks(m.n / 2);
   switch (m.prec) {
-    case 0: mr_update_kernel<double2><<<grid, kVecThreads, 0, st>>>(m); break;
-    case 1: mr_update_kernel<float2><<<grid, kVecThreads, 0, st>>>(m); break;
+    case 0: launch_chain(mr_update_kernel<double2>, grid, kVecThreads, 0, st, m); break;
+    case 1: launch_chain(mr_update_kernel<float2>, grid, kVecThreads, 0, st, m); break;
     case 2:
       if (pairs)
-        mr_update2_kernel<__half2><<<grid, kVecThreads, 0, st>>>(m);
+        launch_chain(mr_update2_kernel<__half2>, grid, kVecThreads, 0, st, m);
       else
-        mr_update_kernel<__half2><<<grid, kVecThreads, 0, st>>>(m);
+        launch_chain(mr_update_kernel<__half2>, grid, kVecThreads, 0, st, m);
       break;
     case 3:
       if (pairs)
-        mr_update2_kernel<__nv_bfloat162><<<grid, kVecThreads, 0, st>>>(m);
+        launch_chain(mr_update2_kernel<__nv_bfloat162>, grid, kVecThreads, 0, st, m);
       else
-        mr_update_kernel<__nv_bfloat162><<<grid, kVecThreads, 0, st>>>(m);
+        launch_chain(mr_update_kernel<__nv_bfloat162>, grid, kVecThreads, 0, st, m);
       break;
     default: return -1;
   }
@@ -154,6 +156,7 @@ int launch_mr_update(const MrUpdate& m, cudaStream_t st) {
 // ------------------------------------------------------------------ dot
 template <typename S>
 __global__ void __launch_bounds__(kVecThreads) dot_kernel(size_t n, const S* a, const S* b, RedArgs ra) {
+  chain_begin();
   typedef typename Store<S>::R R;
   const int rhs = blockIdx.y;
   a += (size_t)rhs * n;
@@ -173,12 +176,11 @@ __global__ void __launch_bounds__(kVecThreads) dot_kernel(size_t n, const S* a, 
 int launch_dot(int prec, size_t n, int nrhs, const void* a, const void* b, RedArgs red, cudaStream_t st) {
   dim3 grid(red_blocks(n), nrhs);
   switch (prec) {
-    case 0: dot_kernel<double2><<<grid, kVecThreads, 0, st>>>(n, (const double2*)a, (const double2*)b, red); break;
-    case 1: dot_kernel<float2><<<grid, kVecThreads, 0, st>>>(n, (const float2*)a, (const float2*)b, red); break;
-    case 2: dot_kernel<__half2><<<grid, kVecThreads, 0, st>>>(n, (const __half2*)a, (const __half2*)b, red); break;
+    case 0: launch_chain(dot_kernel<double2>, grid, kVecThreads, 0, st, n, (const double2*)a, (const double2*)b, red); break;
+    case 1: launch_chain(dot_kernel<float2>, grid, kVecThreads, 0, st, n, (const float2*)a, (const float2*)b, red); break;
+    case 2: launch_chain(dot_kernel<__half2>, grid, kVecThreads, 0, st, n, (const __half2*)a, (const __half2*)b, red); break;
     case 3:
-      dot_kernel<__nv_bfloat162>
-          <<<grid, kVecThreads, 0, st>>>(n, (const __nv_bfloat162*)a, (const __nv_bfloat162*)b, red);
+      launch_chain(dot_kernel<__nv_bfloat162>, grid, kVecThreads, 0, st, n, (const __nv_bfloat162*)a, (const __nv_bfloat162*)b, red);
       break;
     default: return -1;
   }
@@ -210,6 +212,7 @@ template <typename S>
 __global__ void __launch_bounds__(kVecThreads)
     multidot_kernel(size_t n, int k, int kmax, const S* W, size_t jstride, const S* w, RedArgs ra,
                     const double* pre, const double* post, int cstride) {
+  chain_begin();
   typedef typename Store<S>::R R;
   const int chunk = blockIdx.y, rhs = blockIdx.z;
   if (gs_pass_skipped(pre, post, cstride, rhs)) return;
@@ -249,11 +252,11 @@ int launch_multidot(int prec, size_t n, int nrhs, int k, int kmax, const void* W
   dim3 grid(red_blocks(n), (k + kChunk - 1) / kChunk, nrhs);
   switch (prec) {
     case 0:
-      multidot_kernel<double2><<<grid, kVecThreads, 0, st>>>(n, k, kmax, (const double2*)W, jstride, (const double2*)w,
+      launch_chain(multidot_kernel<double2>, grid, kVecThreads, 0, st, n, k, kmax, (const double2*)W, jstride, (const double2*)w,
                                                              red, pre, post, cstride);
       break;
     case 1:
-      multidot_kernel<float2><<<grid, kVecThreads, 0, st>>>(n, k, kmax, (const float2*)W, jstride, (const float2*)w,
+      launch_chain(multidot_kernel<float2>, grid, kVecThreads, 0, st, n, k, kmax, (const float2*)W, jstride, (const float2*)w,
                                                             red, pre, post, cstride);
       break;
     default: return -1;
@@ -265,6 +268,7 @@ template <typename S>
 __global__ void __launch_bounds__(kVecThreads)
     multiaxpy_kernel(size_t n, int k, int kmax, const double* beta, const S* W, const S* Zb, size_t jstride, S* w,
                      S* z, const S* r, RedArgs ra) {
+  chain_begin();
   typedef typename Store<S>::R R;
   __shared__ cx<R> sb[64];
   const int rhs = blockIdx.y;
@@ -311,11 +315,11 @@ int launch_multiaxpy(int prec, size_t n, int nrhs, int k, int kmax, const double
   dim3 grid(vec_blocks(n), nrhs);
   switch (prec) {
     case 0:
-      multiaxpy_kernel<double2><<<grid, kVecThreads, 0, st>>>(n, k, kmax, beta, (const double2*)W, (const double2*)Zb,
+      launch_chain(multiaxpy_kernel<double2>, grid, kVecThreads, 0, st, n, k, kmax, beta, (const double2*)W, (const double2*)Zb,
                                                               jstride, (double2*)w, (double2*)z, (const double2*)r, red2);
       break;
     case 1:
-      multiaxpy_kernel<float2><<<grid, kVecThreads, 0, st>>>(n, k, kmax, beta, (const float2*)W, (const float2*)Zb,
+      launch_chain(multiaxpy_kernel<float2>, grid, kVecThreads, 0, st, n, k, kmax, beta, (const float2*)W, (const float2*)Zb,
                                                              jstride, (float2*)w, (float2*)z, (const float2*)r, red2);
       break;
     default: return -1;
@@ -326,6 +330,7 @@ int launch_multiaxpy(int prec, size_t n, int nrhs, int k, int kmax, const double
 template <typename S, typename SX>
 __global__ void __launch_bounds__(kVecThreads)
     gcr_update_kernel(size_t n, const double* dots, int dstride, S* w, S* z, SX* x, S* r, RedArgs ra) {
+  chain_begin();
   typedef typename Store<S>::R R;
   typedef typename Store<SX>::R RX;
   const int rhs = blockIdx.y;
@@ -370,13 +375,13 @@ int launch_gcr_update(int prec, int xprec, size_t n, int nrhs, const double* dot
                       void* x, void* r, RedArgs red, cudaStream_t st) {
   dim3 grid(vec_blocks(n), nrhs);
   if (prec == 0 && xprec == 0)
-    gcr_update_kernel<double2, double2><<<grid, kVecThreads, 0, st>>>(n, dots, dstride, (double2*)w, (double2*)z,
+    launch_chain(gcr_update_kernel<double2, double2>, grid, kVecThreads, 0, st, n, dots, dstride, (double2*)w, (double2*)z,
                                                                        (double2*)x, (double2*)r, red);
   else if (prec == 1 && xprec == 1)
-    gcr_update_kernel<float2, float2><<<grid, kVecThreads, 0, st>>>(n, dots, dstride, (float2*)w, (float2*)z,
+    launch_chain(gcr_update_kernel<float2, float2>, grid, kVecThreads, 0, st, n, dots, dstride, (float2*)w, (float2*)z,
                                                                      (float2*)x, (float2*)r, red);
   else if (prec == 1 && xprec == 0)
-    gcr_update_kernel<float2, double2><<<grid, kVecThreads, 0, st>>>(n, dots, dstride, (float2*)w, (float2*)z,
+    launch_chain(gcr_update_kernel<float2, double2>, grid, kVecThreads, 0, st, n, dots, dstride, (float2*)w, (float2*)z,
                                                                       (double2*)x, (float2*)r, red);
   else
     return -1;
@@ -398,6 +403,7 @@ template <typename S>
 __global__ void __launch_bounds__(kVecThreads)
     gs_update_kernel(size_t n, int k, int kmax, const double* beta, const S* W, size_t jstride, S* w, const S* r,
                      RedArgs ra, double2* H, int hk, const double* pre, const double* post, int cstride) {
+  chain_begin();
   typedef typename Store<S>::R R;
   __shared__ cx<R> sb[64];
   const int rhs = blockIdx.y;
@@ -441,12 +447,12 @@ int launch_gs_update(int prec, size_t n, int nrhs, int k, int kmax, const double
   dim3 grid(vec_blocks(n), nrhs);
   switch (prec) {
     case 0:
-      gs_update_kernel<double2><<<grid, kVecThreads, 0, st>>>(n, k, kmax, beta, (const double2*)W, jstride,
+      launch_chain(gs_update_kernel<double2>, grid, kVecThreads, 0, st, n, k, kmax, beta, (const double2*)W, jstride,
                                                               (double2*)w, (const double2*)r, red, H, hk, pre, post,
                                                               cstride);
       break;
     case 1:
-      gs_update_kernel<float2><<<grid, kVecThreads, 0, st>>>(n, k, kmax, beta, (const float2*)W, jstride, (float2*)w,
+      launch_chain(gs_update_kernel<float2>, grid, kVecThreads, 0, st, n, k, kmax, beta, (const float2*)W, jstride, (float2*)w,
                                                              (const float2*)r, red, H, hk, pre, post, cstride);
       break;
     default: return -1;
@@ -461,6 +467,7 @@ template <typename S>
 __global__ void __launch_bounds__(kVecThreads)
     gcr_step_kernel(size_t n, const double* dots, int dstride, S* w, S* r, RedArgs ra, double2* H, double2* alpha,
                     int k, int kmax) {
+  chain_begin();
   typedef typename Store<S>::R R;
   const int rhs = blockIdx.y;
   __shared__ double sc[3];
@@ -502,10 +509,10 @@ int launch_gcr_step(int prec, size_t n, int nrhs, const double* dots, int dstrid
                     double2* H, double2* alpha, int k, int kmax, cudaStream_t st) {
   dim3 grid(vec_blocks(n), nrhs);
   if (prec == 0)
-    gcr_step_kernel<double2><<<grid, kVecThreads, 0, st>>>(n, dots, dstride, (double2*)w, (double2*)r, red, H, alpha,
+    launch_chain(gcr_step_kernel<double2>, grid, kVecThreads, 0, st, n, dots, dstride, (double2*)w, (double2*)r, red, H, alpha,
                                                            k, kmax);
   else if (prec == 1)
-    gcr_step_kernel<float2><<<grid, kVecThreads, 0, st>>>(n, dots, dstride, (float2*)w, (float2*)r, red, H, alpha, k,
+    launch_chain(gcr_step_kernel<float2>, grid, kVecThreads, 0, st, n, dots, dstride, (float2*)w, (float2*)r, red, H, alpha, k,
                                                           kmax);
   else
     return -1;
@@ -515,6 +522,7 @@ int launch_gcr_step(int prec, size_t n, int nrhs, const double* dots, int dstrid
 // y = H^-1 alpha for the k x k upper-triangular H of each right-hand side
 // (back substitution in FP64, one thread per right-hand side: k <= 64).
 __global__ void back_substitute_kernel(int k, int kmax, const double2* H, const double2* alpha, double2* y) {
+  chain_begin();
   const int rhs = blockIdx.x;
   if (threadIdx.x != 0) return;
   const double2* Hr = H + (size_t)rhs * kmax * kmax;
@@ -535,7 +543,7 @@ __global__ void back_substitute_kernel(int k, int kmax, const double2* H, const 
 int launch_back_substitute(int nrhs, int k, int kmax, const double2* H, const double2* alpha, double2* y,
                            cudaStream_t st) {
   if (k <= 0) return 0;
-  back_substitute_kernel<<<nrhs, 32, 0, st>>>(k, kmax, H, alpha, y);
+  launch_chain(back_substitute_kernel, nrhs, 32, 0, st, k, kmax, H, alpha, y);
   return launched() ? 0 : -1;
 }
 
@@ -543,6 +551,7 @@ int launch_back_substitute(int nrhs, int k, int kmax, const double2* H, const do
 template <typename SZ, typename SX>
 __global__ void __launch_bounds__(kVecThreads)
     zcombine_kernel(size_t n, int k, int kmax, const double2* y, const SZ* Z, size_t jstride, SX* x) {
+  chain_begin();
   typedef typename Store<SX>::R RX;
   __shared__ cx<RX> sy[64];
   const int rhs = blockIdx.y;
@@ -573,10 +582,10 @@ int launch_zcombine(int zprec, int xprec, size_t n, int nrhs, int k, int kmax, c
   if (k > 64) return -1;
   dim3 grid(vec_blocks(n), nrhs);
   if (zprec == 0 && xprec == 0)
-    zcombine_kernel<double2, double2><<<grid, kVecThreads, 0, st>>>(n, k, kmax, y, (const double2*)Z, jstride,
+    launch_chain(zcombine_kernel<double2, double2>, grid, kVecThreads, 0, st, n, k, kmax, y, (const double2*)Z, jstride,
                                                                     (double2*)x);
   else if (zprec == 1 && xprec == 0)
-    zcombine_kernel<float2, double2><<<grid, kVecThreads, 0, st>>>(n, k, kmax, y, (const float2*)Z, jstride,
+    launch_chain(zcombine_kernel<float2, double2>, grid, kVecThreads, 0, st, n, k, kmax, y, (const float2*)Z, jstride,
                                                                    (double2*)x);
   else
     return -1;
@@ -588,6 +597,7 @@ int launch_zcombine(int zprec, int xprec, size_t n, int nrhs, int k, int kmax, c
 // have a null x; out may be one of the x), with <w|out> and ||out||^2
 // reduced when w is given (lane 0, 3 values).
 __global__ void __launch_bounds__(kVecThreads) lincomb_kernel(size_t n, LinComb L, RedArgs ra) {
+  chain_begin();
   double acc[3] = {0.0, 0.0, 0.0};
   for (size_t i = (size_t)blockIdx.x * kVecThreads + threadIdx.x; i < n; i += (size_t)gridDim.x * kVecThreads) {
     cx<double> v = zero<double>();
@@ -606,7 +616,7 @@ __global__ void __launch_bounds__(kVecThreads) lincomb_kernel(size_t n, LinComb 
 }
 
 int launch_lincomb(size_t n, const LinComb& L, RedArgs red, cudaStream_t st) {
-  lincomb_kernel<<<red_blocks(n), kVecThreads, 0, st>>>(n, L, red);
+  launch_chain(lincomb_kernel, red_blocks(n), kVecThreads, 0, st, n, L, red);
   return launched() ? 0 : -1;
 }
 
@@ -614,6 +624,7 @@ int launch_lincomb(size_t n, const LinComb& L, RedArgs red, cudaStream_t st) {
 template <typename SI, typename SO>
 __global__ void __launch_bounds__(kVecThreads) convert_kernel(size_t n, const SI* in, SO* out, double s0,
                                                               const double* slot, int sstride, double sexp, int acc) {
+  chain_begin();
   const int rhs = blockIdx.y;
   __shared__ double ss;
   if (threadIdx.x == 0) {
@@ -647,12 +658,11 @@ static int convert_to(int pout, dim3 grid, size_t n, const void* in, void* out, 
                       int sstride, double sexp, int acc, cudaStream_t st) {
   const SI* i = (const SI*)in;
   switch (pout) {
-    case 0: convert_kernel<SI, double2><<<grid, kVecThreads, 0, st>>>(n, i, (double2*)out, s0, slot, sstride, sexp, acc); break;
-    case 1: convert_kernel<SI, float2><<<grid, kVecThreads, 0, st>>>(n, i, (float2*)out, s0, slot, sstride, sexp, acc); break;
-    case 2: convert_kernel<SI, __half2><<<grid, kVecThreads, 0, st>>>(n, i, (__half2*)out, s0, slot, sstride, sexp, acc); break;
+    case 0: launch_chain(convert_kernel<SI, double2>, grid, kVecThreads, 0, st, n, i, (double2*)out, s0, slot, sstride, sexp, acc); break;
+    case 1: launch_chain(convert_kernel<SI, float2>, grid, kVecThreads, 0, st, n, i, (float2*)out, s0, slot, sstride, sexp, acc); break;
+    case 2: launch_chain(convert_kernel<SI, __half2>, grid, kVecThreads, 0, st, n, i, (__half2*)out, s0, slot, sstride, sexp, acc); break;
     case 3:
-      convert_kernel<SI, __nv_bfloat162>
-          <<<grid, kVecThreads, 0, st>>>(n, i, (__nv_bfloat162*)out, s0, slot, sstride, sexp, acc);
+      launch_chain(convert_kernel<SI, __nv_bfloat162>, grid, kVecThreads, 0, st, n, i, (__nv_bfloat162*)out, s0, slot, sstride, sexp, acc);
       break;
     default: return -1;
   }

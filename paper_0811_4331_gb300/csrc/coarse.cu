@@ -65,6 +65,7 @@ __device__ __forceinline__ void ld_sites(const S* p, cx<R> (&v)[BV]) {
 // sites, FP64, one (n = 40): 16.5 -> 12.5 us, 12 (n = 48): 97 -> 66.
 template <typename S, int BV, int IR, int RB, int LB>
 __global__ void __launch_bounds__(256) coarse_apply_kernel(const CoarseArgs<S> A, int nrhs) {
+  chain_begin();
   typedef typename Store<S>::R R;
   constexpr int SL = 256 / LB, NO = LB * BV * IR;  // slices; outputs per right-hand side
   __shared__ R part[8 * 2 * NO];  // [warp][re, im][output] of one right-hand side at a time
@@ -202,7 +203,7 @@ static long coarse_ctas(int n, int V, int lb_bv, int ir) {
 template <typename S, int BV, int IR, int RB, int LB>
 static int coarse_go(const CoarseArgs<S>& A, int nrhs, cudaStream_t st) {
   const dim3 grid((unsigned)coarse_ctas(A.n, A.V, LB * BV, IR), (unsigned)((nrhs + RB - 1) / RB));
-  coarse_apply_kernel<S, BV, IR, RB, LB><<<grid, 256, 0, st>>>(A, nrhs);
+  launch_chain(coarse_apply_kernel<S, BV, IR, RB, LB>, grid, 256, 0, st, A, nrhs);
   return launched() ? 0 : -1;
 }
 
@@ -297,6 +298,7 @@ __device__ __forceinline__ int agg_site(const Agg& g, int B, int s) {
 // One CTA per (aggregate, group of NT/32 rows): small coarse grids still fill the GPU.
 template <typename SI, typename SP, typename SO, int NT>
 __global__ void __launch_bounds__(NT) restrict_kernel(const Agg g, const SP* P, const SI* in, SO* out) {
+  chain_begin();
   typedef typename Store<SP>::R R;
   extern __shared__ unsigned char smem_raw[];
   cx<R>* sm = (cx<R>*)smem_raw;  // [ncomp][bsites]
@@ -341,6 +343,7 @@ __global__ void __launch_bounds__(NT) restrict_kernel(const Agg g, const SP* P, 
 // One CTA per (aggregate, group of NT outputs).
 template <typename SI, typename SP, typename SO, int NT>
 __global__ void __launch_bounds__(NT) prolong_kernel(const Agg g, const SP* P, const SI* in, SO* out) {
+  chain_begin();
   typedef typename Store<SP>::R R;
   extern __shared__ unsigned char smem_raw[];
   cx<R>* xc = (cx<R>*)smem_raw;  // [2 nv]
@@ -380,8 +383,7 @@ static int restrict_t(const Agg& g, const void* P, const void* in, void* out, in
   if (sm > 48 * 1024)
     allow_big_smem(restrict_kernel<SI, SP, SO, NT>);
   const int ngroups = (2 * g.nv + NT / 32 - 1) / (NT / 32);
-  restrict_kernel<SI, SP, SO, NT>
-      <<<dim3(g.Vc * ngroups, nrhs), NT, sm, st>>>(g, (const SP*)P, (const SI*)in, (SO*)out);
+  launch_chain(restrict_kernel<SI, SP, SO, NT>, dim3(g.Vc * ngroups, nrhs), NT, sm, st, g, (const SP*)P, (const SI*)in, (SO*)out);
   return launched() ? 0 : -1;
 }
 
@@ -391,8 +393,7 @@ static int prolong_t(const Agg& g, const void* P, const void* in, void* out, int
   constexpr int NT = 256;
   const size_t sm = (size_t)2 * g.nv * sizeof(cx<R>);
   const int ngroups = (g.ncomp * g.bsites + NT - 1) / NT;
-  prolong_kernel<SI, SP, SO, NT>
-      <<<dim3(g.Vc * ngroups, nrhs), NT, sm, st>>>(g, (const SP*)P, (const SI*)in, (SO*)out);
+  launch_chain(prolong_kernel<SI, SP, SO, NT>, dim3(g.Vc * ngroups, nrhs), NT, sm, st, g, (const SP*)P, (const SI*)in, (SO*)out);
   return launched() ? 0 : -1;
 }
 
@@ -628,6 +629,7 @@ template <typename T, int B, int RPT, int NT>
 __global__ void __launch_bounds__(NT) gjb_panel_kernel(T* aug0, int N, int kb, int b, int c1, int n1, int c2,
                                                        int n2, unsigned long long* keys0, int* used0, T* prow0,
                                                        int* err0) {
+  chain_begin();
   typedef typename Store<T>::R R;
   constexpr int LT = B + 1;  // padded row of a warp's staging tile
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -774,6 +776,7 @@ template <typename T>
 __global__ void __launch_bounds__(128) gjb_inner_update_kernel(T* aug0, int N, int kb, int b, int c1, int n1, int c2,
                                                                int n2, const unsigned long long* keys0,
                                                                const T* prow0, const int* err0) {
+  chain_begin();
   typedef typename Store<T>::R R;
   __shared__ cx<R> tes[kGjbRows][8];
   __shared__ int isp[kGjbRows];
@@ -821,6 +824,7 @@ __global__ void __launch_bounds__(128) gjb_inner_update_kernel(T* aug0, int N, i
 template <typename T>
 __global__ void gjb_gather_kernel(const T* aug0, int N, int kb0, int W, const unsigned long long* keys0, T* cp0,
                                   const int* err0) {
+  chain_begin();
   const int z = blockIdx.z;
   if (err0[z]) return;
   const T* aug = aug0 + (size_t)z * N * 2 * N;
@@ -843,6 +847,7 @@ constexpr int kGjTile = 64;
 template <typename T>
 __global__ void __launch_bounds__(256) gjb_outer_update_kernel(T* aug0, int N, int kb0, int W, const int* used0,
                                                                const T* cp0, const int* err0) {
+  chain_begin();
   typedef typename Store<T>::R R;
   constexpr int LA = kGjW + 1;  // padded row of the TE tile
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1004,21 +1009,21 @@ static int dense_inverse_t(const double2* const* C, const int L[4], int n, int b
         const int bw = kb0 + W - kb < b ? kb0 + W - kb : b;
         // the block's columns right of the panel, and the block's earlier slots
         const int c1 = kb + bw, n1 = kb0 + W - c1, c2 = N + kb0, n2 = kb - kb0;
-        panel<<<batch, pnt, psm, st>>>(aug, N, kb, bw, c1, n1, c2, n2, keys, used, prow, err);
+        launch_chain(panel, batch, pnt, psm, st, aug, N, kb, bw, c1, n1, c2, n2, keys, used, prow, err);
         ++nl;
         if (n1 + n2 > 0) {
           const dim3 grid((unsigned)((n1 + n2 + 127) / 128), (unsigned)((N + kGjbRows - 1) / kGjbRows),
                           (unsigned)batch);
-          gjb_inner_update_kernel<T><<<grid, 128, 0, st>>>(aug, N, kb, bw, c1, n1, c2, n2, keys, prow, err);
+          launch_chain(gjb_inner_update_kernel<T>, grid, 128, 0, st, aug, N, kb, bw, c1, n1, c2, n2, keys, prow, err);
           ++nl;
         }
       }
       if (N - W > 0) {
         const dim3 gg((unsigned)((N - W + 255) / 256 < 16 ? (N - W + 255) / 256 : 16), (unsigned)W, (unsigned)batch);
-        gjb_gather_kernel<T><<<gg, 256, 0, st>>>(aug, N, kb0, W, keys, cp, err);
+        launch_chain(gjb_gather_kernel<T>, gg, 256, 0, st, aug, N, kb0, W, keys, cp, err);
         const dim3 go((unsigned)((N - W + kGjTile - 1) / kGjTile), (unsigned)((N + kGjTile - 1) / kGjTile),
                       (unsigned)batch);
-        gjb_outer_update_kernel<T><<<go, 256, smo, st>>>(aug, N, kb0, W, used, cp, err);
+        launch_chain(gjb_outer_update_kernel<T>, go, 256, smo, st, aug, N, kb0, W, used, cp, err);
         nl += 2;
       }
     }
@@ -1078,6 +1083,7 @@ template <typename TM, typename SI, typename SO>
 __global__ void __launch_bounds__(kMmThreads)
     dense_matmul_kernel(int N, const TM* inv, const SI* x, SO* y, int R, int acc, int kper,
                         cx<typename Store<TM>::R>* part, unsigned* tickets) {
+  chain_begin();
   typedef typename Store<TM>::R Rt;
   __shared__ cx<Rt> As[kMmRows][kMmK + 1];
   __shared__ cx<Rt> Bs[kMmK][64];
@@ -1158,6 +1164,7 @@ constexpr int kMvWarps = 4;
 template <typename TM, typename SI, typename SO>
 __global__ void __launch_bounds__(32 * kMvWarps) dense_matvec4_kernel(int N, const TM* inv, const SI* x, SO* y,
                                                                       int acc, const int* midx) {
+  chain_begin();
   typedef typename Store<TM>::R R;
   __shared__ cx<R> part[kMvWarps];
   const int row = blockIdx.x, rhs = blockIdx.y;
@@ -1205,14 +1212,11 @@ int launch_dense_matvec(int pm, int pin, int pout, int N, const void* inv, const
   if (nrhs < 4 || !scratch || midx) {
     const dim3 g((unsigned)N, (unsigned)nrhs);
     if (pm == 0 && pin == 0 && pout == 0)
-      dense_matvec4_kernel<double2, double2, double2>
-          <<<g, 32 * kMvWarps, 0, st>>>(N, (const double2*)inv, (const double2*)x, (double2*)y, acc, midx);
+      launch_chain(dense_matvec4_kernel<double2, double2, double2>, g, 32 * kMvWarps, 0, st, N, (const double2*)inv, (const double2*)x, (double2*)y, acc, midx);
     else if (pm == 1 && pin == 0 && pout == 0)
-      dense_matvec4_kernel<float2, double2, double2>
-          <<<g, 32 * kMvWarps, 0, st>>>(N, (const float2*)inv, (const double2*)x, (double2*)y, acc, midx);
+      launch_chain(dense_matvec4_kernel<float2, double2, double2>, g, 32 * kMvWarps, 0, st, N, (const float2*)inv, (const double2*)x, (double2*)y, acc, midx);
     else if (pm == 1 && pin == 1 && pout == 1)
-      dense_matvec4_kernel<float2, float2, float2>
-          <<<g, 32 * kMvWarps, 0, st>>>(N, (const float2*)inv, (const float2*)x, (float2*)y, acc, midx);
+      launch_chain(dense_matvec4_kernel<float2, float2, float2>, g, 32 * kMvWarps, 0, st, N, (const float2*)inv, (const float2*)x, (float2*)y, acc, midx);
     else
       return -1;
     return launched() ? 0 : -1;
@@ -1227,14 +1231,11 @@ int launch_dense_matvec(int pm, int pin, int pout, int N, const void* inv, const
     const dim3 g(tiles, KS);
     unsigned* tickets = (unsigned*)((char*)scratch + (size_t)8 * 64 * N * 16);
     if (pm == 0 && pin == 0 && pout == 0)
-      dense_matmul_kernel<double2, double2, double2><<<g, kMmThreads, 0, st>>>(
-          N, (const double2*)inv, (const double2*)x, (double2*)y, nrhs, acc, kper, (cx<double>*)scratch, tickets);
+      launch_chain(dense_matmul_kernel<double2, double2, double2>, g, kMmThreads, 0, st, N, (const double2*)inv, (const double2*)x, (double2*)y, nrhs, acc, kper, (cx<double>*)scratch, tickets);
     else if (pm == 1 && pin == 0 && pout == 0)
-      dense_matmul_kernel<float2, double2, double2><<<g, kMmThreads, 0, st>>>(
-          N, (const float2*)inv, (const double2*)x, (double2*)y, nrhs, acc, kper, (cx<float>*)scratch, tickets);
+      launch_chain(dense_matmul_kernel<float2, double2, double2>, g, kMmThreads, 0, st, N, (const float2*)inv, (const double2*)x, (double2*)y, nrhs, acc, kper, (cx<float>*)scratch, tickets);
     else if (pm == 1 && pin == 1 && pout == 1)
-      dense_matmul_kernel<float2, float2, float2><<<g, kMmThreads, 0, st>>>(
-          N, (const float2*)inv, (const float2*)x, (float2*)y, nrhs, acc, kper, (cx<float>*)scratch, tickets);
+      launch_chain(dense_matmul_kernel<float2, float2, float2>, g, kMmThreads, 0, st, N, (const float2*)inv, (const float2*)x, (float2*)y, nrhs, acc, kper, (cx<float>*)scratch, tickets);
     else
       return -1;
     return launched() ? 0 : -1;

@@ -104,6 +104,7 @@ __host__ __device__ constexpr int row_pitch(int npad) { return 4 * npad + 16; }
 // CTA = 32 sites of one right-hand side, transposed through shared memory.
 template <typename S>
 __global__ void __launch_bounds__(256) coarse_rows_kernel(const S* in, unsigned char* rows, int n, int npad, int V, int R) {
+  chain_begin();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int r = blockIdx.y, B0 = blockIdx.x * 32, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int pitch = 4 * npad + 4;  // one bank further per site
@@ -205,6 +206,7 @@ template <typename S, int NT8>
 __global__ void __launch_bounds__(mma_threads(NT8))
     coarse_mma_kernel(const uint4* Cf, const S* in, S* out, const S* y2, int L0, int L1, int L2, int L3, int n, int npad,
                       int R, float a, float c, const double* shift) {
+  chain_begin();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ int nbs[9];
   const int V = L0 * L1 * L2 * L3;
@@ -320,6 +322,7 @@ __global__ void __launch_bounds__(224)
     coarse_stream_kernel(const unsigned char* Cf, const S* in, const unsigned char* rows, S* out, const S* y2, int L0,
                          int L1, int L2, int L3, int n, int npad, int R, float a, float c, const double* shift,
                          int splits, int items, int ns) {
+  chain_begin();
   extern __shared__ __align__(128) unsigned char smem_ring[];
   __shared__ __align__(8) unsigned long long bars[2 * kMaxStages];  // full, empty
   const int V = L0 * L1 * L2 * L3;
@@ -456,9 +459,9 @@ int launch_coarse_mma(int prec, const void* Cf, const void* in, void* out, const
     const size_t smr = (size_t)32 * (4 * npad + 4);
     const dim3 g((unsigned)((V + 31) / 32), (unsigned)R);
     if (prec == 1)
-      coarse_rows_kernel<float2><<<g, 256, smr, st>>>((const float2*)in, rows, n, npad, V, R);
+      launch_chain(coarse_rows_kernel<float2>, g, 256, smr, st, (const float2*)in, rows, n, npad, V, R);
     else
-      coarse_rows_kernel<__nv_bfloat162><<<g, 256, smr, st>>>((const __nv_bfloat162*)in, rows, n, npad, V, R);
+      launch_chain(coarse_rows_kernel<__nv_bfloat162>, g, 256, smr, st, (const __nv_bfloat162*)in, rows, n, npad, V, R);
     if (!launched()) return -1;
   }
   const int items = V * splits;
@@ -470,12 +473,12 @@ int launch_coarse_mma(int prec, const void* Cf, const void* in, void* out, const
   if (rows) {                                                                                               \
     auto kern = coarse_stream_kernel<S, K>;                                                                 \
     allow_big_smem(kern);                                                                                   \
-    kern<<<ctas, 32 * (T + 1), ring, st>>>((const unsigned char*)Cf, (const S*)in, rows, (S*)out, (const S*)y2, L[0], \
+    launch_chain(kern, ctas, 32 * (T + 1), ring, st, (const unsigned char*)Cf, (const S*)in, rows, (S*)out, (const S*)y2, L[0], \
                                            L[1], L[2], L[3], n, npad, R, (float)a, (float)c, shift, splits, items, ns); \
   } else {                                                                                                  \
     auto kern = coarse_mma_kernel<S, K>;                                                                    \
     if (sm > 40 * 1024) allow_big_smem(kern);                                                               \
-    kern<<<dim3(V, splits), 32 * T, sm, st>>>((const uint4*)Cf, (const S*)in, (S*)out, (const S*)y2, L[0], L[1], L[2], \
+    launch_chain(kern, dim3(V, splits), 32 * T, sm, st, (const uint4*)Cf, (const S*)in, (S*)out, (const S*)y2, L[0], L[1], L[2], \
                                               L[3], n, npad, R, (float)a, (float)c, shift);                 \
   }
 #define WMG_MMA_R(S)                       \

@@ -7,6 +7,8 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include <utility>
+
 namespace wmg {
 
 // Launch checks: a launcher reads (and so clears) the thread's last CUDA error
@@ -53,6 +55,39 @@ inline int sm_count() {
     return x;
   }();
   return v;
+}
+
+// Chains of dependent launches.  A kernel of the solver's loops begins with
+// chain_begin(): it waits there until the launches before it on its stream
+// have completed, and lets the next one be launched meanwhile.  Launched with
+// launch_chain it may then start (its blocks take their places, its
+// instructions are fetched) while its predecessor still runs, so a dependent
+// launch costs less than a full drain and start: 18 x 14 x 10 x 21, two MR
+// steps in BF16 (six launches): 49 -> 39 us; 360 launches of a Gauss-Jordan
+// inverse: 6.7 -> 5.9 ms.  Everything after chain_begin() sees its
+// predecessors' memory; a kernel without it is launched with <<<>>>.
+// Not inside a graph capture: a graph's edges cost little by themselves, and
+// there the early blocks took places unevenly (twelve-source solve 309 -> 333
+// ms); nor where a launch of one wave depends on an even placement (the fused
+// setup step, 13.4 -> 14.6 ms of setup).
+__device__ __forceinline__ void chain_begin() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+inline thread_local bool tl_chain_off = false;  // set while this thread captures a graph or solves beside others
+template <typename... P, typename... A>
+inline void launch_chain(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = at;
+  cfg.numAttrs = tl_chain_off ? 0 : 1;
+  cudaLaunchKernelEx(&cfg, kern, std::forward<A>(args)...);  // an error stays for launch_ok()
 }
 
 template <typename K>
@@ -299,25 +334,32 @@ __device__ __forceinline__ void block_sum(T (&v)[NV], T* smem /* NV * NT/32 */) 
   __syncthreads();
 }
 
-// Finish a grid reduction for lane `ln` whose blocks are blockIdx.x in
-// [0, gridDim.x).  Call from every thread of every block with the thread's
-// partial values of type T; NT = blockDim.x (a multiple of 32, <= 1024).
-// The tree inside a block runs in T (FP32 for the FP32 / 16-bit kernels:
-// FP64 arithmetic is scarce on this part); the sum over blocks runs in FP64.
+// The two halves of a grid reduction for lane `ln`: every tile of NT threads'
+// values is summed within its CTA into its own partial (grid_partial), and the
+// last CTA to finish adds the `ntiles` partials in tile order (grid_finish).
+// Call from every thread of every CTA; NT = blockDim.x (a multiple of 32,
+// <= 1024).  The tree inside a tile runs in T (FP32 for the FP32 / 16-bit
+// kernels: FP64 arithmetic is scarce on this part); the sum over tiles runs in
+// FP64.  A CTA may take several tiles before it finishes: the result depends
+// on the tiles alone, not on how CTAs share them.
 template <int NV, int NT, typename T>
-__device__ __forceinline__ void grid_reduce(T (&v)[NV], const RedArgs& ra, int ln) {
+__device__ __forceinline__ void grid_partial(T (&v)[NV], const RedArgs& ra, int ln, int tile, int ntiles) {
   __shared__ T smem_t[NV * (NT / 32)];
-  __shared__ double smem_d[NV * (NT / 32)];
-  __shared__ bool last;
   block_sum<NV, NT, T>(v, smem_t);
-  const int nb = gridDim.x;
   if (threadIdx.x == 0) {
-    double* dst = ra.partials + ((size_t)ln * nb + blockIdx.x) * NV;
+    double* dst = ra.partials + ((size_t)ln * ntiles + tile) * NV;
 #pragma unroll
     for (int k = 0; k < NV; ++k) dst[k] = (double)v[k];
+  }
+}
+template <int NV, int NT>
+__device__ __forceinline__ void grid_finish(const RedArgs& ra, int ln, int ntiles) {
+  __shared__ double smem_d[NV * (NT / 32)];
+  __shared__ bool last;
+  if (threadIdx.x == 0) {
     __threadfence();
     unsigned t = atomicAdd(ra.tickets + ln, 1u);
-    last = (t == (unsigned)nb - 1);
+    last = (t == gridDim.x - 1);
   }
   __syncthreads();
   if (!last) return;
@@ -325,8 +367,8 @@ __device__ __forceinline__ void grid_reduce(T (&v)[NV], const RedArgs& ra, int l
   double w[NV];
 #pragma unroll
   for (int k = 0; k < NV; ++k) w[k] = 0.0;
-  for (int b = threadIdx.x; b < nb; b += NT) {
-    const double* src = ra.partials + ((size_t)ln * nb + b) * NV;
+  for (int b = threadIdx.x; b < ntiles; b += NT) {
+    const double* src = ra.partials + ((size_t)ln * ntiles + b) * NV;
 #pragma unroll
     for (int k = 0; k < NV; ++k) w[k] += __ldcg(src + k);
   }
@@ -336,6 +378,12 @@ __device__ __forceinline__ void grid_reduce(T (&v)[NV], const RedArgs& ra, int l
     for (int k = 0; k < NV; ++k) ra.result[(size_t)ln * ra.stride + k] = w[k];
     ra.tickets[ln] = 0u;
   }
+}
+// One tile per CTA.
+template <int NV, int NT, typename T>
+__device__ __forceinline__ void grid_reduce(T (&v)[NV], const RedArgs& ra, int ln) {
+  grid_partial<NV, NT, T>(v, ra, ln, blockIdx.x, gridDim.x);
+  grid_finish<NV, NT>(ra, ln, gridDim.x);
 }
 
 }  // namespace wmg

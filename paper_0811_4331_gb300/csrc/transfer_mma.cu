@@ -95,6 +95,7 @@ constexpr int kTKs = kTK + 8;   // row stride of a staged plane: rows gid = 0..7
 template <typename T, typename SI, typename SO, int NT8>
 __global__ void __launch_bounds__(kTThreads)
     restrict_mma_kernel(const Agg g, const typename MmaT<T>::T2* P, const SI* in, SO* out, int R, int sidx_off) {
+  chain_begin();
   typedef typename MmaT<T>::T2 T2;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int MT = (g.nv + 15) / 16, Mp = MT * 16, NS = 8 / MT;
@@ -204,6 +205,7 @@ __global__ void __launch_bounds__(kTThreads)
 template <typename T, typename SI, typename SO, int NT8>
 __global__ void __launch_bounds__(kTThreads)
     prolong_mma_kernel(const Agg g, const typename MmaT<T>::T2* P, const SI* in, SO* out, int R, int sidx_off) {
+  chain_begin();
   typedef typename MmaT<T>::T2 T2;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int KT = (g.nv + 15) / 16, Kp = KT * 16, Kps = Kp + 8;  // Kps: bank-spread row stride
@@ -365,6 +367,7 @@ template <typename T, typename SO, int MT, int NCHI, int NGT>
 __global__ void __launch_bounds__(128 * NCHI, 4 / NCHI)
     restrict_tile_kernel(const Agg g, const typename MmaT<T>::T2* P, const typename MmaT<T>::T2* in, SO* out, int R,
                          int nsplit, int vrows, int sidx_off) {
+  chain_begin();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int NCH = NCHI + 1, kVRow = tile_vrow(NCH), VROW = NCH * kVRow, NG = NGT ? NGT : 4;
   const int B = blockIdx.x / nsplit, r0 = (blockIdx.x % nsplit) * MT * 16;
@@ -518,6 +521,7 @@ template <typename T, typename SI, int MT, int NTC>
 __global__ void __launch_bounds__(kProlongThreads, 2)
     prolong_tile_kernel(const Agg g, const typename MmaT<T>::T2* P, const SI* in, typename MmaT<T>::T2* out, int R,
                         int nsplit, int stages, int bufs, int sidx_off) {
+  chain_begin();
   typedef typename MmaT<T>::T2 T2;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int B = blockIdx.x / nsplit, r0 = (blockIdx.x % nsplit) * MT * 16;
@@ -736,7 +740,7 @@ static int restrict_tile_t(const Agg& g, const void* P, const void* in, void* ou
   case (M) * 100 + (C) * 10 + (N): {                                                                        \
     auto kern = restrict_tile_kernel<T, SO, M, C, N>;                                                       \
     if (sm > 48 * 1024) allow_big_smem(kern);                                                               \
-    kern<<<grid, 128 * C, sm, st>>>(g, (const T2*)P, (const T2*)in, (SO*)out, nrhs, nsplit, vrows, (int)so); \
+    launch_chain(kern, grid, 128 * C, sm, st, g, (const T2*)P, (const T2*)in, (SO*)out, nrhs, nsplit, vrows, (int)so); \
     break;                                                                                                  \
   }
 #define WMG_RTN(M, C) WMG_RT(M, C, 0) WMG_RT(M, C, 1) WMG_RT(M, C, 2) WMG_RT(M, C, 3) WMG_RT(M, C, 4)
@@ -772,7 +776,7 @@ static int prolong_tile_t(const Agg& g, const void* P, const void* in, void* out
   case (M) * 10 + (N): {                                                                                          \
     auto kern = prolong_tile_kernel<T, SI, M, N>;                                                                 \
     if (sm > 48 * 1024) allow_big_smem(kern);                                                                     \
-    kern<<<grid, kProlongThreads, sm, st>>>(g, (const T2*)P, (const SI*)in, (T2*)out, nrhs, nsplit, sh.stages, have, \
+    launch_chain(kern, grid, kProlongThreads, sm, st, g, (const T2*)P, (const SI*)in, (T2*)out, nrhs, nsplit, sh.stages, have, \
                                             (int)so);                                                             \
     break;                                                                                                        \
   }
@@ -803,7 +807,7 @@ static int restrict_mma_t(const Agg& g, const void* P, const void* in, void* out
   {                                                                                                            \
     auto kern = restrict_mma_kernel<T, SI, SO, K>;                                                             \
     if (sm > 48 * 1024) allow_big_smem(kern);                                                                  \
-    kern<<<grid, kTThreads, sm, st>>>(g, (const typename MmaT<T>::T2*)P, (const SI*)in, (SO*)out, nrhs, (int)so); \
+    launch_chain(kern, grid, kTThreads, sm, st, g, (const typename MmaT<T>::T2*)P, (const SI*)in, (SO*)out, nrhs, (int)so); \
   }
   switch (NT8) {
     case 1: WMG_RM(1); break;
@@ -837,7 +841,7 @@ static int prolong_mma_t(const Agg& g, const void* P, const void* in, void* out,
   {                                                                                                            \
     auto kern = prolong_mma_kernel<T, SI, SO, K>;                                                              \
     if (sm > 48 * 1024) allow_big_smem(kern);                                                                  \
-    kern<<<grid, kTThreads, sm, st>>>(g, (const typename MmaT<T>::T2*)P, (const SI*)in, (SO*)out, nrhs, (int)so); \
+    launch_chain(kern, grid, kTThreads, sm, st, g, (const typename MmaT<T>::T2*)P, (const SI*)in, (SO*)out, nrhs, (int)so); \
   }
   switch (NT8) {
     case 1: WMG_PM(1); break;

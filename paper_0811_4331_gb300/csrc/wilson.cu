@@ -133,8 +133,8 @@ __device__ __forceinline__ void finish_site(const HA& acc, int r, const S* in, S
 // order for any NT and NR, and the dots of right-hand side r are reduced over
 // the same CTAs of NT sites, so a launch shape never changes a result bit.
 // DOTS: the launch reduces <out|z>, ||out||^2; a CTA then takes several tiles
-// of NT sites, because its reduction ends in a fence and an atomic that all
-// its warps wait for.  Without it a thread takes one site and no reduction
+// of NT sites, each with its partial sums, because a CTA's reduction ends in a
+// fence and an atomic that all its warps wait for.  Without it a thread takes one site and no reduction
 // code runs.  WIDE (FP32): the spinors' chunks as 32-byte loads.
 template <typename S, typename G, int NL, int NT, int NR, bool DOTS, bool WIDE>
 __device__ __forceinline__ void wilson_body(const WilsonArgs<S, G, NL>& A) {
@@ -142,31 +142,38 @@ __device__ __forceinline__ void wilson_body(const WilsonArgs<S, G, NL>& A) {
   const int V = A.V;
   const int rhs0 = blockIdx.y * NR;
   const S* in = A.in + rhs0 * A.vstride;
-  R red[NR][3];  // per-thread partial dots in the arithmetic type
+  const int ntiles = (V + NT - 1) / NT;
+  for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    const int s = tile * NT + threadIdx.x;
+    R red[NR][3];  // per-thread partial dots in the arithmetic type
 #pragma unroll
-  for (int r = 0; r < NR; ++r) red[r][0] = red[r][1] = red[r][2] = (R)0;
-  for (int s = blockIdx.x * NT + threadIdx.x; s < V; s += gridDim.x * NT) {
-    int c[4], stride[4];
-    site_coords(s, A.L, c, stride);
-    HopAcc<R, NR> acc;
-    acc.zero();
-    hop_pair<0, NR, WIDE>(acc, A, in, s, c, stride);
-    hop_pair<1, NR, WIDE>(acc, A, in, s, c, stride);
-    hop_pair<2, NR, WIDE>(acc, A, in, s, c, stride);
-    hop_pair<3, NR, WIDE>(acc, A, in, s, c, stride);
-    const R cb = (R)A.b, cc = (R)A.c;
+    for (int r = 0; r < NR; ++r) red[r][0] = red[r][1] = red[r][2] = (R)0;
+    if (!DOTS && s >= V) return;
+    if (s < V) {
+      int c[4], stride[4];
+      site_coords(s, A.L, c, stride);
+      HopAcc<R, NR> acc;
+      acc.zero();
+      hop_pair<0, NR, WIDE>(acc, A, in, s, c, stride);
+      hop_pair<1, NR, WIDE>(acc, A, in, s, c, stride);
+      hop_pair<2, NR, WIDE>(acc, A, in, s, c, stride);
+      hop_pair<3, NR, WIDE>(acc, A, in, s, c, stride);
+      const R cb = (R)A.b, cc = (R)A.c;
 #pragma unroll
-    for (int r = 0; r < NR; ++r) {
-      const R ca = (R)(A.adiag ? A.a * A.adiag[rhs0 + r] : A.a);
-      const size_t ro = (size_t)(rhs0 + r) * A.vstride;
-      finish_site<R, S, WIDE>(acc, r, A.in + ro, A.out + ro, A.y ? A.y + ro : nullptr, DOTS ? A.z + ro : nullptr,
-                        (size_t)V, s, ca, cb, cc, red[r]);
+      for (int r = 0; r < NR; ++r) {
+        const R ca = (R)(A.adiag ? A.a * A.adiag[rhs0 + r] : A.a);
+        const size_t ro = (size_t)(rhs0 + r) * A.vstride;
+        finish_site<R, S, WIDE>(acc, r, A.in + ro, A.out + ro, A.y ? A.y + ro : nullptr, DOTS ? A.z + ro : nullptr,
+                                (size_t)V, s, ca, cb, cc, red[r]);
+      }
     }
     if (!DOTS) return;  // one site per thread
+#pragma unroll
+    for (int r = 0; r < NR; ++r) grid_partial<3, NT, R>(red[r], A.red, rhs0 + r, tile, ntiles);
   }
   if (DOTS) {
 #pragma unroll
-    for (int r = 0; r < NR; ++r) grid_reduce<3, NT, R>(red[r], A.red, rhs0 + r);
+    for (int r = 0; r < NR; ++r) grid_finish<3, NT>(A.red, rhs0 + r, ntiles);
   }
 }
 
@@ -177,7 +184,7 @@ __device__ __forceinline__ void wilson_body(const WilsonArgs<S, G, NL>& A) {
 //   FP32 plain, 16^3 x 32, 12 right-hand sides: - 115, 640 103 (wide loads included)
 //   16-bit plain: 512 135 (384 152, 640 136, 768 138) at 32^3 x 64
 //   two right-hand sides per thread, FP16, 12: - 105, 384 90.5, 512 90.3 (spills)
-//   fused dots, FP16, 12, in several tiles per CTA: - 134, 512 126, 640 131
+//   fused dots, FP16, 12, in several tiles per CTA: - 134, 512 129, 640 134
 // FP64 is bound by its arithmetic pipe at any of them.
 template <typename S, int NR, bool DOTS>
 __host__ __device__ constexpr int wilson_threads() {
@@ -186,6 +193,7 @@ __host__ __device__ constexpr int wilson_threads() {
 
 template <typename S, typename G, int NL, int NT, int NR, bool DOTS, bool WIDE>
 __global__ void __launch_bounds__(NT, wilson_threads<S, NR, DOTS>() / NT) wilson_kernel(const WilsonArgs<S, G, NL> A) {
+  chain_begin();
   wilson_body<S, G, NL, NT, NR, DOTS, WIDE>(A);
 }
 
@@ -270,6 +278,7 @@ __device__ __forceinline__ void warp_hop_sum(const R (&part)[8][24][32], int j, 
 
 template <typename S, typename G, int NL>
 __global__ void __launch_bounds__(256) wilson_small_kernel(const WilsonArgs<S, G, NL> A) {
+  chain_begin();
   typedef typename Store<S>::R R;
   __shared__ R part[8][24][32];  // [hop][real component][site of the CTA]
   const int V = A.V;
@@ -385,6 +394,7 @@ __device__ __forceinline__ void fused_chunk(const MrFuseArgs& F, const ShiftedIn
 // One thread per site and right-hand side (the hop order of the scalar hop).
 template <typename S, typename G, int NL, int NT>
 __global__ void __launch_bounds__(NT) wilson_mr_kernel(const WilsonArgs<S, G, NL> A, const MrFuseArgs F) {
+  chain_begin();
   typedef typename Store<S>::R R;
   const int V = A.V;
   const int s = blockIdx.x * NT + threadIdx.x;
@@ -420,28 +430,12 @@ __global__ void __launch_bounds__(NT) wilson_mr_kernel(const WilsonArgs<S, G, NL
   grid_reduce<3, NT, R>(red, A.red, rhs);
 }
 
-// FP32 (the mixed setup): packed hops, 32-byte loads (WIDE), several tiles of
-// NT sites per CTA, whose coefficient and reduction then cost once.  Bound by
-// latency at the sizes where it runs.  8^3 x 16, 20 candidates: 37.8 -> 29.2 us
-// a step.  (Forming A r' as p - c A p halves the loads and took 28.5 us, but p's
+// FP32 (the mixed setup): the same operations with 32-byte loads (WIDE) and
+// several tiles of NT sites per CTA, whose coefficient and last reduction step
+// then cost once; the null vectors keep their bits.  Bound by latency at the
+// sizes where it runs.  8^3 x 16, 20 candidates: 37.8 -> 31 us a step.
+// (Forming A r' as p - c A p halves the loads and took 28.5 us, but p's
 // recursion left the null vectors ten times further from 64 bits.)
-template <int MU, typename R, typename S, typename G, int NL, bool WIDE>
-__device__ __forceinline__ void mr_hop_pair(HopAcc<R, 1>& acc, const WilsonArgs<S, G, NL>& A,
-                                            const ShiftedIn<R, S, WIDE>& in, int s, const int (&c)[4],
-                                            const int (&stride)[4]) {
-  const int L = A.L[MU], st = stride[MU];
-  const int fwd = (c[MU] == L - 1) ? s - (L - 1) * st : s + st;
-  const int bwd = (c[MU] == 0) ? s + (L - 1) * st : s - st;
-  Link<R> u;
-  cx<R> psi[12];
-  load_link<R, G, NL>(u, A.U, MU, A.V, s);
-  in(fwd, psi);
-  acc.template add<MU, true>(0, psi, u);
-  load_link<R, G, NL>(u, A.U, MU, A.V, bwd);
-  in(bwd, psi);
-  acc.template add<MU, false>(0, psi, u);
-}
-
 constexpr int kMrThreads = 512;  // per SM (640 spills: 35.9 us)
 template <typename S, typename G, int NL, int NT, bool WIDE>
 __global__ void __launch_bounds__(NT, kMrThreads / NT)
@@ -452,30 +446,43 @@ __global__ void __launch_bounds__(NT, kMrThreads / NT)
   const cx<R> cf = fused_coef<R>(F, rhs);
   const size_t ro = (size_t)rhs * A.vstride;
   const ShiftedIn<R, S, WIDE> in{A.in + ro, (const S*)F.pprev + ro, (size_t)V, cf};
-  R red[3] = {(R)0, (R)0, (R)0};
-  for (int s = blockIdx.x * NT + threadIdx.x; s < V; s += gridDim.x * NT) {
-    int c[4], stride[4];
-    site_coords(s, A.L, c, stride);
-    HopAcc<R, 1> acc;
-    acc.zero();
-    mr_hop_pair<0, R, S, G, NL, WIDE>(acc, A, in, s, c, stride);
-    mr_hop_pair<1, R, S, G, NL, WIDE>(acc, A, in, s, c, stride);
-    mr_hop_pair<2, R, S, G, NL, WIDE>(acc, A, in, s, c, stride);
-    mr_hop_pair<3, R, S, G, NL, WIDE>(acc, A, in, s, c, stride);
+  const int ntiles = (V + NT - 1) / NT;
+  for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    const int s = tile * NT + threadIdx.x;
+    R red[3] = {(R)0, (R)0, (R)0};
+    if (s < V) {
+      int c[4], stride[4];
+      site_coords(s, A.L, c, stride);
+      cx<R> acc[4][3];
 #pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      cx<R> h[4];
+      for (int sp = 0; sp < 4; ++sp)
 #pragma unroll
-      for (int k = 0; k < 4; ++k) h[k] = acc.get(0, 4 * j + k);
-      fused_chunk<R, S, WIDE>(F, in, A.out + ro, ro, j, s, h, (R)A.a, (R)A.b, red);
+        for (int a = 0; a < 3; ++a) acc[sp][a] = zero<R>();
+      one_hop<0, true, R, G, NL>(acc, A.U, V, in, s, c, stride, A.L[0]);
+      one_hop<0, false, R, G, NL>(acc, A.U, V, in, s, c, stride, A.L[0]);
+      one_hop<1, true, R, G, NL>(acc, A.U, V, in, s, c, stride, A.L[1]);
+      one_hop<1, false, R, G, NL>(acc, A.U, V, in, s, c, stride, A.L[1]);
+      one_hop<2, true, R, G, NL>(acc, A.U, V, in, s, c, stride, A.L[2]);
+      one_hop<2, false, R, G, NL>(acc, A.U, V, in, s, c, stride, A.L[2]);
+      one_hop<3, true, R, G, NL>(acc, A.U, V, in, s, c, stride, A.L[3]);
+      one_hop<3, false, R, G, NL>(acc, A.U, V, in, s, c, stride, A.L[3]);
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {
+        cx<R> h[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) h[k] = acc[(4 * j + k) / 3][(4 * j + k) % 3];
+        fused_chunk<R, S, WIDE>(F, in, A.out + ro, ro, j, s, h, (R)A.a, (R)A.b, red);
+      }
     }
+    grid_partial<3, NT, R>(red, A.red, rhs, tile, ntiles);
   }
-  grid_reduce<3, NT, R>(red, A.red, rhs);
+  grid_finish<3, NT>(A.red, rhs, ntiles);
 }
 
 // Small lattices: the warp-per-hop layout of wilson_small_kernel.
 template <typename S, typename G, int NL>
 __global__ void __launch_bounds__(256) wilson_small_mr_kernel(const WilsonArgs<S, G, NL> A, const MrFuseArgs F) {
+  chain_begin();
   typedef typename Store<S>::R R;
   __shared__ R part[8][24][32];
   const int V = A.V;
@@ -499,9 +506,11 @@ __global__ void __launch_bounds__(256) wilson_small_mr_kernel(const WilsonArgs<S
 // Tiles per CTA of a launch with fused dots, of which an SM holds `per_sm` CTAs:
 // CTAs of at most about 16 (FP32) or 4 (16-bit) tiles that fill whole waves, so
 // that few tiles pay for a reduction and none waits for a nearly empty last
-// wave; one tile where 16-bit launches have less than eight waves.  (A function
-// of type and sizes alone: every shape of a launch has the same.)  16^3 x 32, 12 right-hand sides, one tile -> 4 / 8 / 16: FP16 134 ->
-// 125.5 / 134 / 136 us, FP32 181 -> 189 / 161 / 150 us.
+// wave; one tile where 16-bit launches have less than eight waves.  Each tile
+// keeps its own partial sums, so the result does not depend on the choice.
+// 16^3 x 32, 12 right-hand sides, one tile per CTA -> this: FP16 134 -> 129 us,
+// FP32 181 -> 155 (one partial per CTA instead: 124 and 148, but the null
+// vectors' last bits moved, and with them 16-bit roundings of P).
 static int dot_tiles(unsigned tiles, int nrhs, int per_sm, size_t elem) {
   const size_t total = (size_t)tiles * nrhs, slots = (size_t)per_sm * sm_count();
   size_t waves = total / (slots * (elem == 8 ? 16 : 4));
@@ -527,10 +536,10 @@ static int launch_mr_t(const DslashCall& d, const MrFuseArgs& F, cudaStream_t st
   A.red = d.red;
   A.adiag = nullptr;
   if constexpr (NL == 9) {
-    wilson_mr_kernel<S, G, NL, 128><<<dim3((A.V + 127) / 128, d.nrhs), 128, 0, st>>>(A, F);
+    launch_chain(wilson_mr_kernel<S, G, NL, 128>, dim3((A.V + 127) / 128, d.nrhs), 128, 0, st, A, F);
   } else {
     if ((size_t)A.V * d.nrhs <= (size_t)kSmallSites) {  // the same split as the unfused stencil
-      wilson_small_mr_kernel<S, G, NL><<<dim3((A.V + 31) / 32, d.nrhs), 256, 0, st>>>(A, F);
+      launch_chain(wilson_small_mr_kernel<S, G, NL>, dim3((A.V + 31) / 32, d.nrhs), 256, 0, st, A, F);
       return launch_ok() ? 0 : -1;
     }
     constexpr int NT = 128;
@@ -552,12 +561,12 @@ static int launch_nt(const WilsonArgs<S, G, NL>& A, int nrhs, cudaStream_t st) {
     if constexpr (NT == 128) {  // the only CTA size of the dots (kShapesDots)
       const int k = dot_tiles(grid.x, nrhs, wilson_threads<S, 1, true>() / NT, sizeof(S));
       grid.x = (grid.x + k - 1) / k;
-      wilson_kernel<S, G, NL, NT, NR, true, WIDE><<<grid, NT, 0, st>>>(A);
+      launch_chain(wilson_kernel<S, G, NL, NT, NR, true, WIDE>, grid, NT, 0, st, A);
     } else {
       return -1;
     }
   } else {
-    wilson_kernel<S, G, NL, NT, NR, false, WIDE><<<grid, NT, 0, st>>>(A);
+    launch_chain(wilson_kernel<S, G, NL, NT, NR, false, WIDE>, grid, NT, 0, st, A);
   }
   return launch_ok() ? 0 : -1;
 }
@@ -600,7 +609,7 @@ static int launch_t(const DslashCall& d, cudaStream_t st) {
   } else {
     if ((size_t)A.V * d.nrhs <= (size_t)kSmallSites) {  // small lattice: a warp per hop
       dim3 grid((A.V + 31) / 32, d.nrhs);
-      wilson_small_kernel<S, G, NL><<<grid, 256, 0, st>>>(A);
+      launch_chain(wilson_small_kernel<S, G, NL>, grid, 256, 0, st, A);
       return launch_ok() ? 0 : -1;
     }
     WShape sh = {128, 1};

@@ -81,6 +81,7 @@ __device__ __forceinline__ void eo_hop_pair(HopAcc<R, 1>& acc, const EoArgs<S, G
 // 102, FP32 (32-byte loads) 144 -> 129.
 template <typename S, typename G, int NL, int NT, bool DOTS, bool WIDE>
 __global__ void __launch_bounds__(NT, (sizeof(S) == 16 ? 256 : 512) / NT) wilson_eo_kernel(const EoArgs<S, G, NL> A) {
+  chain_begin();
   typedef typename Store<S>::R R;
   const int h = blockIdx.x * NT + threadIdx.x;
   const int rhs = blockIdx.y;
@@ -137,9 +138,9 @@ template <typename S, typename G, int NL, bool WIDE>
 static int launch_eo_w(const EoArgs<S, G, NL>& A, int nrhs, cudaStream_t st) {
   const dim3 grid(eo_blocks(A.V), nrhs);
   if (A.z)
-    wilson_eo_kernel<S, G, NL, kEoThreads, true, WIDE><<<grid, kEoThreads, 0, st>>>(A);
+    launch_chain(wilson_eo_kernel<S, G, NL, kEoThreads, true, WIDE>, grid, kEoThreads, 0, st, A);
   else
-    wilson_eo_kernel<S, G, NL, kEoThreads, false, WIDE><<<grid, kEoThreads, 0, st>>>(A);
+    launch_chain(wilson_eo_kernel<S, G, NL, kEoThreads, false, WIDE>, grid, kEoThreads, 0, st, A);
   return launched() ? 0 : -1;
 }
 
@@ -185,6 +186,7 @@ int launch_wilson_eo(const EoCall& d, cudaStream_t st) {
 template <typename T>
 __global__ void eo_split_kernel(const T* __restrict__ full, T* __restrict__ even, T* __restrict__ odd, int L0, int L1,
                                 int L2, int Vh, size_t hstride) {
+  chain_begin();
   const int h = blockIdx.x * blockDim.x + threadIdx.x;
   if (h >= Vh) return;
   const size_t row = blockIdx.y;
@@ -205,6 +207,7 @@ __global__ void eo_split_kernel(const T* __restrict__ full, T* __restrict__ even
 template <typename S>
 __global__ void eo_merge_kernel(const S* __restrict__ even, const S* __restrict__ odd, S* full, int L0, int L1, int L2,
                                 int Vh, int add) {
+  chain_begin();
   typedef typename Store<S>::R R;
   const int h = blockIdx.x * blockDim.x + threadIdx.x;
   if (h >= Vh) return;
@@ -245,7 +248,7 @@ static int split_t(const void* full, void* even, void* odd, const int L[4], size
                    cudaStream_t st) {
   const int Vh = L[0] * L[1] * L[2] * L[3] / 2;
   dim3 grid((Vh + 255) / 256, (unsigned)rows);
-  eo_split_kernel<T><<<grid, 256, 0, st>>>((const T*)full, (T*)even, (T*)odd, L[0], L[1], L[2], Vh, hstride);
+  launch_chain(eo_split_kernel<T>, grid, 256, 0, st, (const T*)full, (T*)even, (T*)odd, L[0], L[1], L[2], Vh, hstride);
   return launched() ? 0 : -1;
 }
 
@@ -289,7 +292,7 @@ static int merge_t(const void* even, const void* odd, void* full, const int L[4]
                    cudaStream_t st) {
   const int Vh = L[0] * L[1] * L[2] * L[3] / 2;
   dim3 grid((Vh + 255) / 256, (unsigned)rows);
-  eo_merge_kernel<S><<<grid, 256, 0, st>>>((const S*)even, (const S*)odd, (S*)full, L[0], L[1], L[2], Vh, add);
+  launch_chain(eo_merge_kernel<S>, grid, 256, 0, st, (const S*)even, (const S*)odd, (S*)full, L[0], L[1], L[2], Vh, add);
   return launched() ? 0 : -1;
 }
 
