@@ -205,11 +205,13 @@ std::map<std::string, TuneEntry> g_tune;
 int g_tune_mode = 1;
 const int kTuneReps = 3;
 
-template <class F>
-int tuned(mg_handle* h, const std::string& key, int nvar, F&& run) {
+// `key` is called only when there is a choice to look up.
+template <class K, class F>
+int tuned(mg_handle* h, K&& key_of, int nvar, F&& run) {
   if (nvar <= 1 || g_tune_mode == 0) return -1;
   if (g_tune_mode == 3) return nvar - 1;
   if (g_tune_mode == 4) return 0;
+  const std::string key = key_of();
   std::lock_guard<std::mutex> lk(g_tune_mu);
   auto it = g_tune.find(key);
   if (it != g_tune.end()) return it->second.variant;
@@ -283,7 +285,7 @@ int op_apply(mg_handle* h, int l, int prec, const void* in, void* out, const voi
     const double lb = 4.0 * a.V * (prec == MG_F64 ? 9 : 6) * bytes_of(prec);
     {
       DevBuf scratch;
-      d.variant = tuned(h, tkey("dslash", {prec, a.L[0], a.L[1], a.L[2], a.L[3], nrhs, y != nullptr, z != nullptr}),
+      d.variant = tuned(h, [&] { return tkey("dslash", {prec, a.L[0], a.L[1], a.L[2], a.L[3], nrhs, y != nullptr, z != nullptr}); },
                         wilson_variants(prec, z != nullptr, nrhs, a.V), [&](int v) {
                           if (!scratch.p && !scratch.ensure((size_t)a.n() * nrhs * bytes_of(prec))) return -1;
                           DslashCall t = d;
@@ -308,7 +310,7 @@ int op_apply(mg_handle* h, int l, int prec, const void* in, void* out, const voi
     }
     {
       DevBuf scratch;
-      const int var = tuned(h, tkey("coarse_mma", {prec, a.ncomp, a.V, nrhs}), coarse_mma_variants(nrhs), [&](int v) {
+      const int var = tuned(h, [&] { return tkey("coarse_mma", {prec, a.ncomp, a.V, nrhs}); }, coarse_mma_variants(nrhs), [&](int v) {
         if (!scratch.p && !scratch.ensure((size_t)vb * nrhs)) return -1;
         return launch_coarse_mma(prec, a.cop_mma.p, in, scratch.p, y, a.L, a.ncomp, nrhs, a_, c_, h->st, v, mmshift,
                                  rows);
@@ -666,12 +668,12 @@ int vcycle(mg_handle* h, int l, const void* r, void* e, int nrhs) {
   if (xmma) {
     DevBuf scratch;
     const size_t need = (size_t)std::max(fbytes, cbytes);
-    rvar = tuned(h, tkey("restrict_mma", {prec, pc, a.nv, a.bsites, a.Vc, nrhs}), transfer_mma_variants(g, nrhs, false),
+    rvar = tuned(h, [&] { return tkey("restrict_mma", {prec, pc, a.nv, a.bsites, a.Vc, nrhs}); }, transfer_mma_variants(g, nrhs, false),
                  [&](int v) {
                    if (!scratch.p && !scratch.ensure(need)) return -1;
                    return launch_restrict(prec, prec, pc, g, a.P[prec].p, res, scratch.p, nrhs, h->st, v);
                  });
-    pvar = tuned(h, tkey("prolong_mma", {prec, pc, a.nv, a.bsites, a.Vc, nrhs}), transfer_mma_variants(g, nrhs, true),
+    pvar = tuned(h, [&] { return tkey("prolong_mma", {prec, pc, a.nv, a.bsites, a.Vc, nrhs}); }, transfer_mma_variants(g, nrhs, true),
                  [&](int v) {
                    if (!scratch.p && !scratch.ensure(need)) return -1;
                    return launch_prolong(pc, prec, prec, g, a.P[prec].p, rc, scratch.p, nrhs, h->st, v);
