@@ -208,12 +208,45 @@ __device__ __forceinline__ bool gs_pass_skipped(const double* pre, const double*
   return !(post[(size_t)rhs * cstride] < 0.5 * pre[(size_t)rhs * cstride]);
 }
 
+// Sum of 16 values per lane over the warp: lane l returns the total of value
+// l / 2.  Each step halves the values a lane keeps while it halves the lanes, so
+// it takes 16 shuffles instead of 80; every total is the same tree.
+template <typename R>
+__device__ __forceinline__ R warp_sum16(const R (&v)[16]) {
+  const int lane = threadIdx.x & 31;
+  R a[8], b[4], c[2], d;
+  const bool h4 = lane & 16, h3 = lane & 8, h2 = lane & 4, h1 = lane & 2;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) a[i] = (h4 ? v[i + 8] : v[i]) + __shfl_xor_sync(0xffffffffu, h4 ? v[i] : v[i + 8], 16);
+#pragma unroll
+  for (int i = 0; i < 4; ++i) b[i] = (h3 ? a[i + 4] : a[i]) + __shfl_xor_sync(0xffffffffu, h3 ? a[i] : a[i + 4], 8);
+#pragma unroll
+  for (int i = 0; i < 2; ++i) c[i] = (h2 ? b[i + 2] : b[i]) + __shfl_xor_sync(0xffffffffu, h2 ? b[i] : b[i + 2], 4);
+  d = (h1 ? c[1] : c[0]) + __shfl_xor_sync(0xffffffffu, h1 ? c[0] : c[1], 2);
+  return d + __shfl_xor_sync(0xffffffffu, d, 1);
+}
+
+// Blocks per chunk and right-hand side: at least 4 elements per thread, at most one block per SM.
+static int multidot_blocks(size_t n) {
+  const size_t b = (n + 4 * kVecThreads - 1) / (4 * kVecThreads);
+  const size_t cap = (size_t)sm_count() < (size_t)kMaxVecBlocks ? (size_t)sm_count() : (size_t)kMaxVecBlocks;
+  return (int)(b > cap ? cap : (b < 1 ? 1 : b));
+}
+
+// On small lattices the reduction of the 16 sums was most of the time (a tree of
+// FP64 additions per value in the last block): 8^3 x 16 (98,304 elements), up to
+// 8 vectors, 18.5 -> 6.8 us.
 template <typename S>
 __global__ void __launch_bounds__(kVecThreads)
     multidot_kernel(size_t n, int k, int kmax, const S* W, size_t jstride, const S* w, RedArgs ra,
                     const double* pre, const double* post, int cstride) {
   chain_begin();
   typedef typename Store<S>::R R;
+  constexpr int NV = 2 * kChunk, NW = kVecThreads / 32, NG = kVecThreads / NV;
+  static_assert(NV == 16, "warp_sum16");
+  __shared__ R sw[NV][NW];
+  __shared__ double sg[NG][NV];
+  __shared__ bool last;
   const int chunk = blockIdx.y, rhs = blockIdx.z;
   if (gs_pass_skipped(pre, post, cstride, rhs)) return;
   const int j0 = chunk * kChunk;
@@ -222,6 +255,7 @@ __global__ void __launch_bounds__(kVecThreads)
   cx<R> acc[kChunk];
 #pragma unroll
   for (int q = 0; q < kChunk; ++q) acc[q] = zero<R>();
+#pragma unroll 2
   for (size_t i = (size_t)blockIdx.x * kVecThreads + threadIdx.x; i < n; i += (size_t)gridDim.x * kVecThreads) {
     const cx<R> x = ldc<R>(wr, i);
     cx<R> v[kChunk];
@@ -230,34 +264,58 @@ __global__ void __launch_bounds__(kVecThreads)
 #pragma unroll
     for (int q = 0; q < kChunk; ++q) acc[q] = cfma_conj(v[q], x, acc[q]);
   }
-  R red[2 * kChunk];
+  R red[NV];
 #pragma unroll
   for (int q = 0; q < kChunk; ++q) {
     red[2 * q] = acc[q].re;
     red[2 * q + 1] = acc[q].im;
   }
-  // lane = rhs * nchunks + chunk; the result is laid out so that beta_j of
-  // rhs r sits at result[(r * kmax + j) * 2]: stride between lanes is 2 CH
-  // within one rhs, 2 kmax between rhs.
-  RedArgs r2 = ra;
-  r2.result = ra.result + (size_t)rhs * kmax * 2 + (size_t)chunk * 2 * kChunk - (size_t)(rhs * gridDim.y + chunk) * 2 * kChunk;
-  r2.stride = 2 * kChunk;
-  grid_reduce<2 * kChunk, kVecThreads, R>(red, r2, rhs * gridDim.y + chunk);
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const R ws = warp_sum16<R>(red);
+  if (!(lane & 1)) sw[lane >> 1][warp] = ws;
+  __syncthreads();
+  // lane of the reduction = rhs * nchunks + chunk, its partials [block][16]
+  const int ln = rhs * gridDim.y + chunk, nb = gridDim.x;
+  double* part = ra.partials + (size_t)ln * nb * NV;
+  if (t < NV) {
+    R s = sw[t][0];
+#pragma unroll
+    for (int u = 1; u < NW; ++u) s += sw[t][u];
+    part[(size_t)blockIdx.x * NV + t] = (double)s;
+  }
+  __syncthreads();
+  if (t == 0) last = take_ticket(ra.tickets + ln) == (unsigned)nb - 1;
+  __syncthreads();
+  if (!last) return;
+  // thread = value t % 16 of blocks t / 16, t / 16 + 16, ...; then the groups in order
+  double s = 0.0;
+#pragma unroll 4
+  for (int b = t / NV; b < nb; b += NG) s += __ldcg(part + (size_t)b * NV + t % NV);
+  sg[t / NV][t % NV] = s;
+  __syncthreads();
+  if (t < NV) {
+    double r = sg[0][t];
+#pragma unroll
+    for (int u = 1; u < NG; ++u) r += sg[u][t];
+    // beta_j of rhs r sits at result[(r * kmax + j) * 2]
+    ra.result[(size_t)rhs * kmax * 2 + (size_t)chunk * NV + t] = r;
+  }
+  if (t == 0) ra.tickets[ln] = 0u;
 }
 
 int launch_multidot(int prec, size_t n, int nrhs, int k, int kmax, const void* W, size_t jstride, const void* w,
                     RedArgs red, cudaStream_t st, const double* pre, const double* post, int cstride) {
   if (k <= 0) return 0;
   if (kmax % kChunk) return -1;
-  dim3 grid(red_blocks(n), (k + kChunk - 1) / kChunk, nrhs);
+  dim3 grid(multidot_blocks(n), (k + kChunk - 1) / kChunk, nrhs);
   switch (prec) {
     case 0:
-      launch_chain(multidot_kernel<double2>, grid, kVecThreads, 0, st, n, k, kmax, (const double2*)W, jstride, (const double2*)w,
-                                                             red, pre, post, cstride);
+      launch_chain(multidot_kernel<double2>, grid, kVecThreads, 0, st, n, k, kmax, (const double2*)W, jstride,
+                   (const double2*)w, red, pre, post, cstride);
       break;
     case 1:
-      launch_chain(multidot_kernel<float2>, grid, kVecThreads, 0, st, n, k, kmax, (const float2*)W, jstride, (const float2*)w,
-                                                            red, pre, post, cstride);
+      launch_chain(multidot_kernel<float2>, grid, kVecThreads, 0, st, n, k, kmax, (const float2*)W, jstride,
+                   (const float2*)w, red, pre, post, cstride);
       break;
     default: return -1;
   }
@@ -519,25 +577,35 @@ int launch_gcr_step(int prec, size_t n, int nrhs, const double* dots, int dstrid
   return launched() ? 0 : -1;
 }
 
-// y = H^-1 alpha for the k x k upper-triangular H of each right-hand side
-// (back substitution in FP64, one thread per right-hand side: k <= 64).
+// y = H^-1 alpha for the k x k upper-triangular H of each right-hand side: back
+// substitution in FP64 by one warp per right-hand side (k <= 64), row i's sum
+// over its lanes' columns.  8^3 x 16, 20 to 25 vectors: one thread took 74 us, the warp 41.
 __global__ void back_substitute_kernel(int k, int kmax, const double2* H, const double2* alpha, double2* y) {
   chain_begin();
-  const int rhs = blockIdx.x;
-  if (threadIdx.x != 0) return;
+  __shared__ double2 ys[64];
+  const int rhs = blockIdx.x, lane = threadIdx.x;
   const double2* Hr = H + (size_t)rhs * kmax * kmax;
   const double2* ar = alpha + (size_t)rhs * kmax;
-  double2* yr = y + (size_t)rhs * kmax;
   for (int i = k - 1; i >= 0; --i) {
-    double sr = ar[i].x, si = ar[i].y;
-    for (int j = i + 1; j < k; ++j) {
-      const double2 h = Hr[(size_t)i * kmax + j], v = yr[j];
-      sr -= h.x * v.x - h.y * v.y;
-      si -= h.x * v.y + h.y * v.x;
+    double sr = 0.0, si = 0.0;
+    for (int j = i + 1 + lane; j < k; j += 32) {
+      const double2 h = Hr[(size_t)i * kmax + j], v = ys[j];
+      sr += h.x * v.x - h.y * v.y;
+      si += h.x * v.y + h.y * v.x;
     }
-    const double dd = Hr[(size_t)i * kmax + i].x;
-    yr[i] = dd > 0.0 ? make_double2(sr / dd, si / dd) : make_double2(0.0, 0.0);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      sr += __shfl_xor_sync(0xffffffffu, sr, o);
+      si += __shfl_xor_sync(0xffffffffu, si, o);
+    }
+    if (lane == 0) {
+      const double dd = Hr[(size_t)i * kmax + i].x;
+      const double2 r = make_double2(ar[i].x - sr, ar[i].y - si);
+      ys[i] = dd > 0.0 ? make_double2(r.x / dd, r.y / dd) : make_double2(0.0, 0.0);
+    }
+    __syncwarp();
   }
+  for (int j = lane; j < k; j += 32) y[(size_t)rhs * kmax + j] = ys[j];
 }
 
 int launch_back_substitute(int nrhs, int k, int kmax, const double2* H, const double2* alpha, double2* y,

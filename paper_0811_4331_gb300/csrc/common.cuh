@@ -352,18 +352,22 @@ __device__ __forceinline__ void grid_partial(T (&v)[NV], const RedArgs& ra, int 
     for (int k = 0; k < NV; ++k) dst[k] = (double)v[k];
   }
 }
+// Next ticket of a counter, releasing this thread's earlier writes (and those it
+// has seen through a barrier) and acquiring those of the earlier tickets.  One
+// instruction, and weaker than the two sequentially consistent fences around a
+// plain atomic.
+__device__ __forceinline__ unsigned take_ticket(unsigned* t) {
+  unsigned v;
+  asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(v) : "l"(t) : "memory");
+  return v;
+}
 template <int NV, int NT>
 __device__ __forceinline__ void grid_finish(const RedArgs& ra, int ln, int ntiles) {
   __shared__ double smem_d[NV * (NT / 32)];
   __shared__ bool last;
-  if (threadIdx.x == 0) {
-    __threadfence();
-    unsigned t = atomicAdd(ra.tickets + ln, 1u);
-    last = (t == gridDim.x - 1);
-  }
+  if (threadIdx.x == 0) last = take_ticket(ra.tickets + ln) == gridDim.x - 1;
   __syncthreads();
   if (!last) return;
-  __threadfence();
   double w[NV];
 #pragma unroll
   for (int k = 0; k < NV; ++k) w[k] = 0.0;
