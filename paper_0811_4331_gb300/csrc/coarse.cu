@@ -1156,70 +1156,128 @@ size_t dense_matvec_scratch_bytes(int N) {
   return (size_t)8 * 64 * N * 16 + (size_t)((N + kMmRows - 1) / kMmRows) * sizeof(unsigned) + 256;
 }
 
-// y = inv x (+ y if acc) for 1-3 right-hand sides: a CTA of kMvWarps warps per
-// row, warp w summing columns [w N / kMvWarps, (w+1) N / kMvWarps) with two
-// independent chains, the warps' sums added in warp order (deterministic).
-constexpr int kMvWarps = 4;
+// y = inv x (+ y if acc) for a few right-hand sides, or with a matrix per
+// right-hand side (midx, RB = 1).  CTA = kMvRows rows (two warps each, halves of
+// the columns) and RB right-hand sides, whose vectors it first stages in the
+// matrix's precision: a conversion from FP64 runs on the scarce FP64 pipe, and
+// one per row and column was half of the time.  The matrix is read in 16-byte
+// pieces, four in flight per lane; warp sums in a fixed order.
+// N = 1280, FP32 inverse, one right-hand side: 9.0 -> 6.1 us.
+constexpr int kMvRows = 4, kMvThreads = 64 * kMvRows;
 
-template <typename TM, typename SI, typename SO>
-__global__ void __launch_bounds__(32 * kMvWarps) dense_matvec4_kernel(int N, const TM* inv, const SI* x, SO* y,
-                                                                      int acc, const int* midx) {
+template <typename TM, typename SI, typename SO, int RB>
+__global__ void __launch_bounds__(kMvThreads) dense_matvec_kernel(int N, const TM* inv, const SI* x, SO* y, int nrhs,
+                                                                  int acc, const int* midx) {
   chain_begin();
   typedef typename Store<TM>::R R;
-  __shared__ cx<R> part[kMvWarps];
-  const int row = blockIdx.x, rhs = blockIdx.y;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int c0 = (int)((long)warp * N / kMvWarps), c1 = (int)((long)(warp + 1) * N / kMvWarps);
-  const TM* rp = inv + (midx ? (size_t)midx[rhs] * N * N : (size_t)0) + (size_t)row * N;
-  const SI* xr = x + (size_t)rhs * N;
-  cx<R> a = zero<R>(), b = zero<R>();
-  int j = c0 + lane;
-  // eight loads in flight per lane; chain a takes columns j, j + 64, ..., chain b j + 32, j + 96, ...
-  for (; j + 96 < c1; j += 128) {
-    const cx<R> m0 = ldc<R>(rp, j), m1 = ldc<R>(rp, j + 32), m2 = ldc<R>(rp, j + 64), m3 = ldc<R>(rp, j + 96);
-    const cx<R> x0 = ldc<R>(xr, j), x1 = ldc<R>(xr, j + 32), x2 = ldc<R>(xr, j + 64), x3 = ldc<R>(xr, j + 96);
-    a = cfma(m0, x0, a);
-    b = cfma(m1, x1, b);
-    a = cfma(m2, x2, a);
-    b = cfma(m3, x3, b);
+  constexpr int E = (int)(16 / sizeof(TM));  // matrix elements per 16 bytes
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  cx<R>* xs = (cx<R>*)smem_raw;  // [RB][N]
+  __shared__ cx<R> part[kMvRows][2][RB];
+  const int r0 = blockIdx.y * RB, rows = min(RB, nrhs - r0);
+  for (int e = threadIdx.x; e < RB * N; e += kMvThreads) {
+    const int r = RB == 1 ? 0 : e / N;
+    xs[e] = r < rows ? ldc<R>(x, (size_t)r0 * N + e) : zero<R>();
   }
-  for (; j + 32 < c1; j += 64) {
-    a = cfma(ldc<R>(rp, j), ldc<R>(xr, j), a);
-    b = cfma(ldc<R>(rp, j + 32), ldc<R>(xr, j + 32), b);
-  }
-  for (; j < c1; j += 32) a = cfma(ldc<R>(rp, j), ldc<R>(xr, j), a);
-  a = a + b;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    a.re += __shfl_down_sync(0xffffffffu, a.re, o);
-    a.im += __shfl_down_sync(0xffffffffu, a.im, o);
-  }
-  if (lane == 0) part[warp] = a;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    cx<R> s = part[0];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, half = warp & 1;
+  const int row = blockIdx.x * kMvRows + (warp >> 1);
+  const int mid = (N / 2 + E - 1) / E * E, c0 = half ? mid : 0, c1 = half ? N : mid;
+  cx<R> a[RB];
 #pragma unroll
-    for (int w = 1; w < kMvWarps; ++w) s = s + part[w];
-    const size_t o = (size_t)rhs * N + row;
-    cx<double> v = mk<double>((double)s.re, (double)s.im);
-    if (acc) v = v + ldc<double>(y, o);
-    stc(y, o, v);
+  for (int r = 0; r < RB; ++r) a[r] = zero<R>();
+  if (row < N) {
+    const TM* rp = inv + (midx ? (size_t)midx[r0] * N * N : (size_t)0) + (size_t)row * N;
+    auto fma_col = [&](const cx<R>& m, int j) {
+#pragma unroll
+      for (int r = 0; r < RB; ++r) a[r] = cfma(m, xs[r * N + j], a[r]);
+    };
+    int j = c0;
+    if (E == 1 || N % E == 0) {  // rows start on 16 bytes
+      auto load = [&](int at, cx<R> (&m)[E]) {
+        if constexpr (E == 1) {
+          m[0] = ldc<R>(rp, at);
+        } else {
+          const float4 q = __ldg(reinterpret_cast<const float4*>(rp + at));
+          m[0] = mk<R>(q.x, q.y);
+          m[1] = mk<R>(q.z, q.w);
+        }
+      };
+      for (; j + 4 * 32 * E <= c1; j += 4 * 32 * E) {
+        cx<R> m[4][E];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) load(j + (u * 32 + lane) * E, m[u]);
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+          for (int q = 0; q < E; ++q) fma_col(m[u][q], j + (u * 32 + lane) * E + q);
+      }
+    }
+    for (j += lane; j < c1; j += 32) fma_col(ldc<R>(rp, j), j);
+  }
+#pragma unroll
+  for (int r = 0; r < RB; ++r) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      a[r].re += __shfl_down_sync(0xffffffffu, a[r].re, o);
+      a[r].im += __shfl_down_sync(0xffffffffu, a[r].im, o);
+    }
+    if (lane == 0) part[warp >> 1][half][r] = a[r];
+  }
+  __syncthreads();
+  if (threadIdx.x < kMvRows * RB) {
+    const int q = threadIdx.x % kMvRows, r = threadIdx.x / kMvRows, i = blockIdx.x * kMvRows + q;
+    if (i < N && r < rows) {
+      const cx<R> s = part[q][0][r] + part[q][1][r];
+      const size_t o = (size_t)(r0 + r) * N + i;
+      cx<double> v = mk<double>((double)s.re, (double)s.im);
+      if (acc) v = v + ldc<double>(y, o);
+      stc(y, o, v);
+    }
   }
 }
 
+template <typename TM, typename SI, typename SO>
+static int matvec_go(int N, const void* inv, const void* x, void* y, int nrhs, int acc, const int* midx,
+                     cudaStream_t st) {
+  typedef typename Store<TM>::R R;
+  const unsigned gx = (unsigned)((N + kMvRows - 1) / kMvRows);
+  constexpr int kRB = sizeof(R) == 8 ? 2 : 4;
+  const size_t most = (size_t)smem_optin_bytes() - 2048;
+  const bool one = nrhs == 1 || midx || (size_t)kRB * N * sizeof(cx<R>) > most;
+  const size_t sm = (size_t)(one ? 1 : kRB) * N * sizeof(cx<R>);
+  if (sm > most) return -1;  // above 8192 rows, which no hierarchy has
+#define WMG_MV(B)                                                                                                 \
+  {                                                                                                               \
+    auto kern = dense_matvec_kernel<TM, SI, SO, B>;                                                               \
+    if (sm > 40 * 1024) allow_big_smem(kern);                                                                     \
+    launch_chain(kern, dim3(gx, (unsigned)((nrhs + B - 1) / B)), kMvThreads, sm, st, N, (const TM*)inv, (const SI*)x, \
+                 (SO*)y, nrhs, acc, midx);                                                                        \
+  }
+  if (one)
+    WMG_MV(1)
+  else
+    WMG_MV(kRB)
+#undef WMG_MV
+  return launched() ? 0 : -1;
+}
+
+// Right-hand sides up to which the row form runs: it reads the matrix once per
+// four, the tiled product once (N = 1536: 12 right-hand sides 36 us against 53,
+// 24 61 against 60; N = 768, 48: 33 against 27).
+constexpr int kMvMost = 16;
+
 int launch_dense_matvec(int pm, int pin, int pout, int N, const void* inv, const void* x, void* y, int nrhs, int acc,
                         cudaStream_t st, void* scratch, const int* midx) {
-  if (nrhs < 4 || !scratch || midx) {
-    const dim3 g((unsigned)N, (unsigned)nrhs);
+  if (nrhs <= kMvMost || !scratch || midx) {
+    int rc = -1;
     if (pm == 0 && pin == 0 && pout == 0)
-      launch_chain(dense_matvec4_kernel<double2, double2, double2>, g, 32 * kMvWarps, 0, st, N, (const double2*)inv, (const double2*)x, (double2*)y, acc, midx);
+      rc = matvec_go<double2, double2, double2>(N, inv, x, y, nrhs, acc, midx, st);
     else if (pm == 1 && pin == 0 && pout == 0)
-      launch_chain(dense_matvec4_kernel<float2, double2, double2>, g, 32 * kMvWarps, 0, st, N, (const float2*)inv, (const double2*)x, (double2*)y, acc, midx);
+      rc = matvec_go<float2, double2, double2>(N, inv, x, y, nrhs, acc, midx, st);
     else if (pm == 1 && pin == 1 && pout == 1)
-      launch_chain(dense_matvec4_kernel<float2, float2, float2>, g, 32 * kMvWarps, 0, st, N, (const float2*)inv, (const float2*)x, (float2*)y, acc, midx);
-    else
-      return -1;
-    return launched() ? 0 : -1;
+      rc = matvec_go<float2, float2, float2>(N, inv, x, y, nrhs, acc, midx, st);
+    return rc;
   }
   if (scratch && nrhs >= 4 && nrhs <= 64) {
     const int tiles = (N + kMmRows - 1) / kMmRows;
