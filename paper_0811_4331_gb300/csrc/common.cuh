@@ -352,6 +352,47 @@ __device__ __forceinline__ void grid_partial(T (&v)[NV], const RedArgs& ra, int 
     for (int k = 0; k < NV; ++k) dst[k] = (double)v[k];
   }
 }
+// Sums of lane ln's `ntiles` partials, valid in thread 0: thread t takes the
+// partials t, t + NT, ..., and the threads' sums are added in the tree of
+// block_sum, but level by level through shared memory with every lane at work.
+// A warp's FP64 addition occupies this part's FP64 unit whether one lane needs
+// it or 32: the shuffle tree issues 135 of them for three values and 256
+// threads, this about 25, and the last block of a reduction waits for them
+// (18 x 14 x 10 x 21, two BF16 MR steps: 41 -> 39 us).  The same bits.
+template <int NV, int NT>
+__device__ __forceinline__ void sum_partials(double (&w)[NV], const double* partials, int ln, int ntiles,
+                                             double* smem /* NV * NT */) {
+#pragma unroll
+  for (int k = 0; k < NV; ++k) w[k] = 0.0;
+  for (int b = threadIdx.x; b < ntiles; b += NT) {
+    const double* src = partials + ((size_t)ln * ntiles + b) * NV;
+#pragma unroll
+    for (int k = 0; k < NV; ++k) w[k] += __ldcg(src + k);
+  }
+#pragma unroll
+  for (int k = 0; k < NV; ++k) smem[k * NT + threadIdx.x] = w[k];
+  __syncthreads();
+  // within groups of 32: element i of a group takes element i + o
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    for (int e = threadIdx.x; e < NV * (NT / 32) * o; e += NT) {
+      double* q = smem + (e / o) * 32 + e % o;
+      *q += q[o];
+    }
+    __syncthreads();
+  }
+  // the groups' sums
+#pragma unroll
+  for (int o = NT / 64; o > 0; o >>= 1) {
+    if ((int)threadIdx.x < NV * o) {
+      double* q = smem + (threadIdx.x / o) * NT + (threadIdx.x % o) * 32;
+      *q += q[o * 32];
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int k = 0; k < NV; ++k) w[k] = smem[k * NT];
+}
 // Next ticket of a counter, releasing this thread's earlier writes (and those it
 // has seen through a barrier) and acquiring those of the earlier tickets.  One
 // instruction, and weaker than the two sequentially consistent fences around a
@@ -363,20 +404,13 @@ __device__ __forceinline__ unsigned take_ticket(unsigned* t) {
 }
 template <int NV, int NT>
 __device__ __forceinline__ void grid_finish(const RedArgs& ra, int ln, int ntiles) {
-  __shared__ double smem_d[NV * (NT / 32)];
+  __shared__ double smem_d[NV * NT];
   __shared__ bool last;
   if (threadIdx.x == 0) last = take_ticket(ra.tickets + ln) == gridDim.x - 1;
   __syncthreads();
   if (!last) return;
   double w[NV];
-#pragma unroll
-  for (int k = 0; k < NV; ++k) w[k] = 0.0;
-  for (int b = threadIdx.x; b < ntiles; b += NT) {
-    const double* src = ra.partials + ((size_t)ln * ntiles + b) * NV;
-#pragma unroll
-    for (int k = 0; k < NV; ++k) w[k] += __ldcg(src + k);
-  }
-  block_sum<NV, NT, double>(w, smem_d);
+  sum_partials<NV, NT>(w, ra.partials, ln, ntiles, smem_d);
   if (threadIdx.x == 0) {
 #pragma unroll
     for (int k = 0; k < NV; ++k) ra.result[(size_t)ln * ra.stride + k] = w[k];
