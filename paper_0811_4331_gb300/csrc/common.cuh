@@ -362,6 +362,7 @@ __device__ __forceinline__ void grid_partial(T (&v)[NV], const RedArgs& ra, int 
 template <int NV, int NT>
 __device__ __forceinline__ void sum_partials(double (&w)[NV], const double* partials, int ln, int ntiles,
                                              double* smem /* NV * NT */) {
+  static_assert((NT & (NT - 1)) == 0 && NT >= 32, "the tree halves NT");
 #pragma unroll
   for (int k = 0; k < NV; ++k) w[k] = 0.0;
   for (int b = threadIdx.x; b < ntiles; b += NT) {
@@ -405,10 +406,10 @@ __device__ __forceinline__ unsigned take_ticket(unsigned* t) {
 template <int NV, int NT>
 __device__ __forceinline__ void grid_finish(const RedArgs& ra, int ln, int ntiles) {
   __shared__ double smem_d[NV * NT];
-  __shared__ bool last;
-  if (threadIdx.x == 0) last = take_ticket(ra.tickets + ln) == gridDim.x - 1;
-  __syncthreads();
-  if (!last) return;
+  // the barrier carries the flag: a CTA may finish several lanes in turn, and a
+  // flag in shared memory could be overwritten before every warp has read it
+  const bool mine = threadIdx.x == 0 && take_ticket(ra.tickets + ln) == gridDim.x - 1;
+  if (!__syncthreads_or(mine)) return;
   double w[NV];
   sum_partials<NV, NT>(w, ra.partials, ln, ntiles, smem_d);
   if (threadIdx.x == 0) {
