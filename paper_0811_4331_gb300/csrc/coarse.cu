@@ -61,8 +61,9 @@ __device__ __forceinline__ void ld_sites(const S* p, cx<R> (&v)[BV]) {
 // CTA (deterministic).  With one right-hand side the operator's bytes bound it
 // (85 MB on 512 sites, n = 48, FP32), with several in FP64 the FP64 pipe.
 // The operator is read once per RB right-hand sides.
-// 512 sites, n = 48, FP32, one right-hand side: 33 -> 20.7 us, 12: 243 -> 77; 32
-// sites, FP64, one (n = 40): 16.5 -> 12.5 us, 12 (n = 48): 97 -> 66.
+// 512 sites, n = 48, FP32, one right-hand side: 33 -> 20.7 us (18 with
+// chained launches), 12: 243 -> 77; 32 sites, FP64, one (n = 40): 16.5 -> 12.5
+// us, 12 (n = 48): 97 -> 66.
 template <typename S, int BV, int IR, int RB, int LB>
 __global__ void __launch_bounds__(256) coarse_apply_kernel(const CoarseArgs<S> A, int nrhs) {
   chain_begin();

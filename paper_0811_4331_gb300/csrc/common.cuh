@@ -63,7 +63,7 @@ inline int sm_count() {
 // launch_chain it may then start (its blocks take their places, its
 // instructions are fetched) while its predecessor still runs, so a dependent
 // launch costs less than a full drain and start: 18 x 14 x 10 x 21, two MR
-// steps in BF16 (six launches): 49 -> 39 us; 360 launches of a Gauss-Jordan
+// steps in BF16 (six launches): 49 -> 41 us; 360 launches of a Gauss-Jordan
 // inverse: 6.7 -> 5.9 ms.  Everything after chain_begin() sees its
 // predecessors' memory; a kernel without it is launched with <<<>>>.
 // Not inside a graph capture: a graph's edges cost little by themselves, and

@@ -300,8 +300,8 @@ __global__ void __launch_bounds__(kTThreads)
 // consecutive aggregate sites, which is how they lie in memory: a lane reads
 // a site's two components as 8 bytes, and writes a site's chunk as 16.
 //
-// 16^3 x 32, nv = 24, 24 right-hand sides, FP16: restriction 211 -> 66 us,
-// prolongation 226 -> 66 us (4.6 TB/s; 45 us is the floor).
+// 16^3 x 32, nv = 24, 24 right-hand sides, FP16: restriction 212 -> 64 us,
+// prolongation 226 -> 64.5 us (4.8 TB/s; 45 us is the floor).
 constexpr int kTileE = 16;                     // sites per stage
 constexpr int kTilePRow = 6 * kTileE * 4 + 16;  // bytes of a staged row of P (4 mod 32 words: no bank conflicts)
 // ... and of a staged (right-hand side, chunk): nch = 3 or 2 of them per right-hand side are 64 mod 128

@@ -77,8 +77,8 @@ __device__ __forceinline__ void eo_hop_pair(HopAcc<R, 1>& acc, const EoArgs<S, G
 // One thread per half site and right-hand side, packed hops and the register
 // budget of the full stencil (512 threads per SM; 640 and 768, and two
 // right-hand sides per thread at 384 to 512, are 1-5 % slower).  S (two
-// launches) on 16^3 x 32, 12 right-hand sides: FP16 117 -> 110 us, BF16 118 ->
-// 102, FP32 (32-byte loads) 144 -> 129.
+// launches) on 16^3 x 32, 12 right-hand sides: FP16 117 -> 111 us (106
+// with chained launches), BF16 118 -> 102, FP32 (32-byte loads) 144 -> 129.
 template <typename S, typename G, int NL, int NT, bool DOTS, bool WIDE>
 __global__ void __launch_bounds__(NT, (sizeof(S) == 16 ? 256 : 512) / NT) wilson_eo_kernel(const EoArgs<S, G, NL> A) {
   chain_begin();
