@@ -92,10 +92,12 @@ __device__ __forceinline__ void ld_chunk(const S* p, size_t i, cx<R> (&v)[4]) {
 }
 // Four FP32 complex elements as one 32-byte load (p + i on a 32-byte boundary):
 // a warp's load is then one contiguous 1 KB run instead of two half-used ones.
+// volatile: chain_begin()'s wait is a volatile asm too, and only among those is
+// the order kept; otherwise a load might move up before the predecessor's end.
 template <typename R>
 __device__ __forceinline__ void ld_chunk_wide(const float2* p, size_t i, cx<R> (&v)[4]) {
   float f[8];
-  asm("ld.global.nc.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+  asm volatile("ld.global.nc.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
       : "=f"(f[0]), "=f"(f[1]), "=f"(f[2]), "=f"(f[3]), "=f"(f[4]), "=f"(f[5]), "=f"(f[6]), "=f"(f[7])
       : "l"(p + i));
 #pragma unroll
