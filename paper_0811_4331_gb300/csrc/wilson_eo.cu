@@ -183,9 +183,10 @@ int launch_wilson_eo(const EoCall& d, cudaStream_t st) {
 // and one odd site (the parity of 2h is that of y + z + t).  Rows are
 // right-hand side x component (or mu x link element); the halves of row r
 // start at even + r * hstride and odd + r * hstride.
+// (No __restrict__ here and below: loads through it count as invariant over the
+// whole kernel and could be moved above chain_begin()'s wait.)
 template <typename T>
-__global__ void eo_split_kernel(const T* __restrict__ full, T* __restrict__ even, T* __restrict__ odd, int L0, int L1,
-                                int L2, int Vh, size_t hstride) {
+__global__ void eo_split_kernel(const T* full, T* even, T* odd, int L0, int L1, int L2, int Vh, size_t hstride) {
   chain_begin();
   const int h = blockIdx.x * blockDim.x + threadIdx.x;
   if (h >= Vh) return;
@@ -205,8 +206,7 @@ __global__ void eo_split_kernel(const T* __restrict__ full, T* __restrict__ even
 // full = (add ? full : 0) + merge(even, odd) on chunked level-0 fields (rows
 // of V four-component chunks); a null half is zero.
 template <typename S>
-__global__ void eo_merge_kernel(const S* __restrict__ even, const S* __restrict__ odd, S* full, int L0, int L1, int L2,
-                                int Vh, int add) {
+__global__ void eo_merge_kernel(const S* even, const S* odd, S* full, int L0, int L1, int L2, int Vh, int add) {
   chain_begin();
   typedef typename Store<S>::R R;
   const int h = blockIdx.x * blockDim.x + threadIdx.x;
