@@ -744,10 +744,8 @@ int vcycle_graph(mg_handle* h, const void* r, void* e, int nrhs) {
     std::shared_lock<std::shared_mutex> nosync(g_capture_mu);
     ce = cudaStreamBeginCapture(h->cap_st, cudaStreamCaptureModeThreadLocal);
     if (ce == cudaSuccess) {
-      const bool chain_off = tl_chain_off;
-      tl_chain_off = true;  // see launch_chain
+      const ChainOff chain_off(true);  // see launch_chain
       rc = vcycle(h, 0, r, e, nrhs);
-      tl_chain_off = chain_off;
       ce = cudaStreamEndCapture(h->cap_st, &graph);
     }
   }
@@ -2556,11 +2554,7 @@ extern "C" int mg_solve_many(mg_handle* const* hs, int count, const double* cons
   auto run = [&](int i) {
     // side by side, early blocks of one solve take the other solves' places (four 8^3 x 16 solves: 16.7 ms without
     // launch_chain's early starts, 17.1 with)
-    struct ChainOff {
-      bool prev = tl_chain_off;
-      explicit ChainOff(bool off) { tl_chain_off = prev || off; }
-      ~ChainOff() { tl_chain_off = prev; }
-    } chain_off(count > 1);
+    const ChainOff chain_off(count > 1);
     cudaStream_t st = streams ? (cudaStream_t)streams[i] : nullptr;
     bool own = false;
     if (!st) {

@@ -11,8 +11,6 @@
 // site of the aggregate in x-fastest order): the restriction of one coarse
 // component is a contiguous dot product and the prolongation of one fine
 // component a contiguous column read.
-#include <algorithm>
-
 #include "common.cuh"
 #include "kernels.h"
 
@@ -53,9 +51,9 @@ __device__ __forceinline__ void ld_sites(const S* p, cx<R> (&v)[BV]) {
   }
 }
 
-// CTA = LB x BV consecutive sites, IR rows i and RB right-hand sides; its 256
-// threads are LB groups of BV sites times 256 / LB slices of the 9 n terms
-// (d, j).  A thread reads BV sites of a matrix element as one 16-byte load for
+// CTA = LB consecutive units (BV sites of IR rows i each, `pitch` units per IR
+// rows: launch_rules.h) and RB right-hand sides; its 256 threads are the LB units
+// times 256 / LB slices of the 9 n terms (d, j).  A thread reads BV sites of a matrix element as one 16-byte load for
 // each of its IR rows, and the neighbour's component once for all of them;
 // the slices are added by shuffles within a warp and in warp order across the
 // CTA (deterministic).  With one right-hand side the operator's bytes bound it
@@ -65,23 +63,28 @@ __device__ __forceinline__ void ld_sites(const S* p, cx<R> (&v)[BV]) {
 // chained launches), 12: 243 -> 77; 32 sites, FP64, one (n = 40): 16.5 -> 12.5
 // us, 12 (n = 48): 97 -> 66.
 template <typename S, int BV, int IR, int RB, int LB>
-__global__ void __launch_bounds__(256) coarse_apply_kernel(const CoarseArgs<S> A, int nrhs) {
+__global__ void 
+    __launch_bounds__(256, sizeof(S) == 8 && BV == 2 && IR * RB == 2 ? 3 : 0)  // two registers above three per SM
+    coarse_apply_kernel(const CoarseArgs<S> A, int pitch, int nrhs) {
   chain_begin();
   typedef typename Store<S>::R R;
   constexpr int SL = 256 / LB, NO = LB * BV * IR;  // slices; outputs per right-hand side
   __shared__ R part[8 * 2 * NO];  // [warp][re, im][output] of one right-hand side at a time
-  __shared__ int nbs[9][LB * BV];
+  __shared__ int nbs[9][LB * BV];  // a unit's sites (direction 0) and their neighbours
+  __shared__ int rows[LB];         // a unit's first row, n if it has no sites
   const int V = A.V, n = A.n;
-  const int nbb = (V + LB * BV - 1) / (LB * BV);
-  const int Bc = (blockIdx.x % nbb) * LB * BV, i0 = (blockIdx.x / nbb) * IR, r0 = blockIdx.y * RB;
+  const int r0 = blockIdx.y * RB;
   const int bl = threadIdx.x % LB, sl = threadIdx.x / LB;
-  for (int e = threadIdx.x; e < 9 * LB * BV; e += 256) {
-    const int d = e / (LB * BV), b = e - d * LB * BV;
+  if (threadIdx.x < LB * BV) {
+    const int u = blockIdx.x * LB + threadIdx.x / BV, ib = u / pitch, B = (u - ib * pitch) * BV + threadIdx.x % BV;
     int c[4];
-    site_coords(min(Bc + b, V - 1), A.L, c);
-    nbs[d][b] = neighbor(c, A.L, d);
+    site_coords(min(B, V - 1), A.L, c);
+#pragma unroll
+    for (int d = 0; d < 9; ++d) nbs[d][threadIdx.x] = neighbor(c, A.L, d);
+    if (threadIdx.x % BV == 0) rows[threadIdx.x / BV] = B < V ? min(ib * IR, n) : n;
   }
   __syncthreads();
+  const int i0 = rows[bl];
   cx<R> acc[RB][IR][BV];
 #pragma unroll
   for (int r = 0; r < RB; ++r)
@@ -89,8 +92,8 @@ __global__ void __launch_bounds__(256) coarse_apply_kernel(const CoarseArgs<S> A
     for (int i = 0; i < IR; ++i)
 #pragma unroll
       for (int v = 0; v < BV; ++v) acc[r][i][v] = zero<R>();
-  const int B0 = Bc + bl * BV;
-  if (B0 < V) {
+  if (i0 < n) {
+    const int B0 = nbs[0][bl * BV];
     // rows past n and right-hand sides past the last repeat the last one; neither is stored
     const S* Ci[IR];
     const S* xr[RB];
@@ -162,8 +165,8 @@ __global__ void __launch_bounds__(256) coarse_apply_kernel(const CoarseArgs<S> A
     red[r][0] = red[r][1] = red[r][2] = (R)0;
 #pragma unroll
     for (int o = threadIdx.x; o < NO; o += 256) {
-      const int B = Bc + (o % LB) * BV + (o / LB) % BV, i = i0 + o / (LB * BV);
-      if (B >= V || i >= n || r0 + r >= nrhs) continue;
+      const int B = nbs[0][o % LB * BV + o / LB % BV], i = rows[o % LB] + o / (LB * BV);
+      if (i >= n || r0 + r >= nrhs) continue;
       cx<R> s = zero<R>();
 #pragma unroll
       for (int w = 0; w < 8; ++w) s = s + mk<R>(part[w * 2 * NO + o], part[w * 2 * NO + NO + o]);
@@ -188,45 +191,30 @@ __global__ void __launch_bounds__(256) coarse_apply_kernel(const CoarseArgs<S> A
   }
 }
 
-// Tile of a launch.  Up to kCoarseLarge outputs: 16 site groups and the most
-// rows (4, 2, 1) that leave two CTAs per SM -- rows share the vector's loads,
-// but few CTAs leave the GPU idle (32 sites, n = 48, 12 right-hand sides, FP32:
-// 10.6 us with one row, 16.7 with four; 512 sites: 103 with two, 76 with four;
-// one right-hand side 20.7 with two, 27.8 with one).  FP64 takes one row: it is
-// bound by its arithmetic and wants CTAs, and no lane for a right-hand side that is
-// not there.  Above, 32 site groups, and for one right-hand side rows enough to
-// keep the reduction partials few.
-constexpr long kCoarseLarge = 65536;
-static long coarse_ctas(int n, int V, int lb_bv, int ir) {
-  return (long)((V + lb_bv - 1) / lb_bv) * ((n + ir - 1) / ir);
-}
-
 template <typename S, int BV, int IR, int RB, int LB>
-static int coarse_go(const CoarseArgs<S>& A, int nrhs, cudaStream_t st) {
-  const dim3 grid((unsigned)coarse_ctas(A.n, A.V, LB * BV, IR), (unsigned)((nrhs + RB - 1) / RB));
-  launch_chain(coarse_apply_kernel<S, BV, IR, RB, LB>, grid, 256, 0, st, A, nrhs);
+static int coarse_go(const CoarseArgs<S>& A, long pitch, int nrhs, cudaStream_t st) {
+  const dim3 grid((unsigned)coarse_ctas(A.n, IR, LB, pitch), (unsigned)((nrhs + RB - 1) / RB));
+  // FP64: a CTA more on one SM costs what the others do, so crowded launches wait for their predecessor's end
+  static const int per_sm = sizeof(S) == 16 ? ctas_per_sm(coarse_apply_kernel<S, BV, IR, RB, LB>, 256, 0) : 0;
+  const ChainOff crowded(per_sm && !chain_fits((long)grid.x * grid.y, per_sm, sm_count()));
+  launch_chain(coarse_apply_kernel<S, BV, IR, RB, LB>, grid, 256, 0, st, A, (int)pitch, nrhs);
   return launched() ? 0 : -1;
 }
 
-template <typename S, int BV, int RB>
+// The kernel of a shape (launch_rules.h gives the rule).
+template <typename S, int BV>
 static int coarse_launch(const CoarseArgs<S>& A, int nrhs, cudaStream_t st) {
-  constexpr bool f64 = sizeof(S) == 16;
-  if ((long)A.n * A.V >= kCoarseLarge) {
-    if constexpr (RB == 1)
-      return nrhs == 1 ? coarse_go<S, BV, BV == 1 ? 4 : 2, 1, 32>(A, nrhs, st) : coarse_go<S, BV, 1, 1, 32>(A, nrhs, st);
-    else
-      return coarse_go<S, BV, f64 ? 1 : (RB == 4 ? 4 : 2), RB, 32>(A, nrhs, st);
-  }
-  const long gy = (nrhs + RB - 1) / RB, want = 2L * sm_count();
-  if constexpr (!f64) {
-    if constexpr (RB == 4)
-      if (coarse_ctas(A.n, A.V, 16 * BV, 4) * gy >= want) return coarse_go<S, BV, 4, RB, 16>(A, nrhs, st);
-    if (coarse_ctas(A.n, A.V, 16 * BV, 2) * gy >= want) return coarse_go<S, BV, 2, RB, 16>(A, nrhs, st);
-  } else {
-    // half the slices are half the additions that join them
-    if (coarse_ctas(A.n, A.V, 32, 1) * gy >= 2 * want) return coarse_go<S, BV, 1, RB, 32>(A, nrhs, st);
-  }
-  return coarse_go<S, BV, 1, RB, 16>(A, nrhs, st);
+  const CoarseShape sh = coarse_shape(sizeof(S), A.n, A.V, nrhs, sm_count());
+#define WMG_CO(I, R, B)                                         \
+  if constexpr (coarse_has((int)sizeof(S), BV, I, R, B))        \
+    if (sh.ir == I && sh.rb == R && sh.lb == B) return coarse_go<S, BV, I, R, B>(A, sh.pitch, nrhs, st);
+#define WMG_CO_R(I, R) WMG_CO(I, R, 4) WMG_CO(I, R, 8) WMG_CO(I, R, 16) WMG_CO(I, R, 32)
+#define WMG_CO_I(I) WMG_CO_R(I, 1) WMG_CO_R(I, 2) WMG_CO_R(I, 4)
+  WMG_CO_I(1) WMG_CO_I(2) WMG_CO_I(4)
+#undef WMG_CO_I
+#undef WMG_CO_R
+#undef WMG_CO
+  return -1;
 }
 
 template <typename S>
@@ -245,14 +233,9 @@ static int coarse_launch_s(const CoarseCall& k, int V, cudaStream_t st) {
   A.red = k.red;
   A.shift = k.shift;
   constexpr int BV = (int)(16 / sizeof(S));
-  if constexpr (BV > 1) {
-    if (V % BV != 0)  // a row of sites does not start on 16 bytes
-      return k.nrhs == 1 ? coarse_launch<S, 1, 1>(A, 1, st) : coarse_launch<S, 1, 4>(A, k.nrhs, st);
-  }
-  if (k.nrhs == 1 || (sizeof(S) == 16 && k.nrhs % 2)) return coarse_launch<S, BV, 1>(A, k.nrhs, st);
-  if (k.nrhs == 2 || sizeof(S) == 16) return coarse_launch<S, BV, 2>(A, k.nrhs, st);
-  if constexpr (sizeof(S) < 16) return coarse_launch<S, BV, 4>(A, k.nrhs, st);
-  return -1;
+  if constexpr (BV > 1)
+    if (coarse_bv(sizeof(S), V) == 1) return coarse_launch<S, 1>(A, k.nrhs, st);
+  return coarse_launch<S, BV>(A, k.nrhs, st);
 }
 
 int launch_coarse_apply(const CoarseCall& k, cudaStream_t st) {
@@ -264,23 +247,6 @@ int launch_coarse_apply(const CoarseCall& k, cudaStream_t st) {
     case 3: return coarse_launch_s<__nv_bfloat162>(k, V, st);
   }
   return -1;
-}
-
-// CTAs of a launch per right-hand side, at most (sizes the reduction partials;
-// not below the count this function has always given).
-int coarse_blocks(int ncomp, int V, int nrhs) {
-  const long outs = (long)ncomp * V;
-  long G = 1;
-  while (G < 32 && outs * G < 65536) G *= 2;
-  long most = (outs * G + 127) / 128;
-  long c;
-  if (outs < kCoarseLarge)
-    c = coarse_ctas(ncomp, V, 16, 1);
-  else if (nrhs == 1)
-    c = std::max(coarse_ctas(ncomp, V, 32, 4), V % 2 ? 0L : coarse_ctas(ncomp, V, 64, 2));
-  else
-    c = coarse_ctas(ncomp, V, 32, 1);
-  return (int)(c > most ? c : most);
 }
 
 // ------------------------------------------------------------------ aggregates

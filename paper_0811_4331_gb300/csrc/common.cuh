@@ -75,6 +75,23 @@ __device__ __forceinline__ void chain_begin() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 inline thread_local bool tl_chain_off = false;  // set while this thread captures a graph or solves beside others
+// While alive (and `off`), this thread's launch_chain launches wait for their predecessor's end.
+struct ChainOff {
+  const bool prev = tl_chain_off;
+  explicit ChainOff(bool off) { tl_chain_off = prev || off; }
+  ~ChainOff() { tl_chain_off = prev; }
+  ChainOff(const ChainOff&) = delete;
+};
+// CTAs of a kernel that an SM holds at once (0: not to be had).
+template <typename K>
+inline int ctas_per_sm(K kern, int threads, size_t smem) {
+  int n = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, threads, smem) != cudaSuccess) {
+    cudaGetLastError();
+    n = 0;
+  }
+  return n;
+}
 template <typename... P, typename... A>
 inline void launch_chain(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
   cudaLaunchAttribute at[1];

@@ -8,6 +8,7 @@
 #include <stdint.h>
 
 #include "common.cuh"
+#include "launch_rules.h"
 
 namespace wmg {
 
@@ -185,7 +186,6 @@ struct CoarseCall {
   const double* shift = nullptr;  // per right-hand side: out = a (A + shift[r] 1) in + c y
 };
 int launch_coarse_apply(const CoarseCall& k, cudaStream_t st);
-int coarse_blocks(int ncomp, int V, int nrhs);
 
 // Tensor-core coarse stencil (BF16 mma.sync, FP32 accumulation) for R <= 64
 // right-hand sides of storage prec (1 = FP32, 3 = BF16): out = a A in + c y2.

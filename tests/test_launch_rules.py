@@ -1,0 +1,47 @@
+"""The launch rules (csrc/launch_rules.h, plain C++) over the sizes that hierarchies have, compiled for the host.
+
+- coarse stencil: every tile it picks has a kernel, fits the reduction's partials, and leaves few lanes idle.
+"""
+import os
+import shutil
+import subprocess
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_0811_4331_gb300", "csrc")
+
+
+def _run(tmp_path, body):
+    if not shutil.which("g++"):
+        pytest.skip("g++ not available")
+    src = tmp_path / "rules.cpp"
+    src.write_text("#include <cstdio>\n#include \"launch_rules.h\"\nusing namespace wmg;\nint main() {\n%s\n}\n" % body)
+    exe = tmp_path / "rules"
+    subprocess.run(["g++", "-O1", "-std=c++17", "-Wall", "-Werror", "-I", CSRC, str(src), "-o", str(exe)], check=True)
+    out = subprocess.run([str(exe)], capture_output=True, text=True, check=True).stdout
+    return [tuple(int(x) for x in line.split()) for line in out.splitlines()]
+
+
+def test_coarse_tiles(tmp_path):
+    rows = _run(tmp_path, """
+  const int elems[] = {16, 8, 4};
+  for (int elem : elems)
+    for (long n = 2; n <= 128; n += n < 20 ? 2 : 6)
+      for (long V = 1; V <= 20000; V += V < 130 ? 1 : V / 7)
+        for (int r = 1; r <= 64; r += r < 6 ? 1 : 5) {
+          const CoarseShape s = coarse_shape(elem, n, V, r, 152);
+          const int bv = coarse_bv(elem, V);
+          printf("%d %d %ld %ld %d %d %d %d %ld %ld %ld %d\\n", elem, bv, n, V, r, s.ir, s.rb, s.lb, s.pitch,
+                 coarse_ctas(n, s.ir, s.lb, s.pitch), coarse_blocks(n, V, r),
+                 coarse_has(elem, bv, s.ir, s.rb, s.lb));
+        }""")
+    assert len(rows) > 10000
+    for elem, bv, n, V, r, ir, rb, lb, pitch, ctas, blocks, has in rows:
+        case = (elem, n, V, r)
+        assert has, (case, ir, rb, lb)
+        assert ctas <= blocks, case
+        groups = V // bv
+        assert ctas * lb >= -(-n // ir) * pitch and pitch >= groups, case
+        # lanes: FP64 (bound by arithmetic) idles in the last CTA alone, the others less than a third of a row
+        assert pitch == groups if elem == 16 else 2 * pitch < 3 * groups, case
+        assert pitch == groups or pitch % lb == 0, case
