@@ -97,6 +97,22 @@ inline CoarseShape coarse_shape(size_t elem, long n, long V, int nrhs, int sms) 
   return {1, rb, lb, pitch(lb)};
 }
 
+// ------------------------------------------------------------------ fine stencil
+// Threads an SM is to hold, one thread per site, for elements of `elem` bytes,
+// i.e. the register budget (65,536 / threads).  Measured (us per launch; "-":
+// the compiler's own choice of 96-102, 144 in FP64, 180 for two right-hand sides
+// per thread):
+//   FP32 plain, 32^3 x 64: - 168, 512 170, 640 158, 768 162
+//   FP32 plain, 16^3 x 32, 12 right-hand sides: - 115, 640 103 (wide loads included)
+//   16-bit plain: 512 135 (384 152, 640 136, 768 138) at 32^3 x 64
+//   two right-hand sides per thread, FP16, 12: - 105, 384 90.5, 512 90.3 (spills)
+//   fused dots, FP16, 12, in several tiles per CTA: - 134, 512 129, 640 134
+//   FP64, 9 x 7 x 5 x 11, 12 right-hand sides (336 CTAs): 256 114 (a second wave), 384 101; bound by its arithmetic
+//   pipe, 16^3 x 32 takes 233 with either
+constexpr int stencil_threads(int elem, int nr, bool dots) {
+  return elem == 16 ? 384 : (nr == 2 ? 384 : (elem == 8 && !dots ? 640 : 512));
+}
+
 // ------------------------------------------------------------------ chained launches
 // Whether a launch may start early (launch_chain) without crowding.  The CTAs of
 // an early launch take the places that its predecessor leaves.  A second grid of

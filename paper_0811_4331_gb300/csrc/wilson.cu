@@ -177,18 +177,10 @@ __device__ __forceinline__ void wilson_body(const WilsonArgs<S, G, NL>& A) {
   }
 }
 
-// Threads an SM is to hold, i.e. the register budget (65,536 / threads).
-// Measured (us per launch; "-": the compiler's own choice of 96-102, 180 for
-// two right-hand sides per thread):
-//   FP32 plain, 32^3 x 64: - 168, 512 170, 640 158, 768 162
-//   FP32 plain, 16^3 x 32, 12 right-hand sides: - 115, 640 103 (wide loads included)
-//   16-bit plain: 512 135 (384 152, 640 136, 768 138) at 32^3 x 64
-//   two right-hand sides per thread, FP16, 12: - 105, 384 90.5, 512 90.3 (spills)
-//   fused dots, FP16, 12, in several tiles per CTA: - 134, 512 129, 640 134
-// FP64 is bound by its arithmetic pipe at any of them.
+// Threads an SM is to hold, i.e. the register budget (launch_rules.h).
 template <typename S, int NR, bool DOTS>
 __host__ __device__ constexpr int wilson_threads() {
-  return sizeof(S) == 16 ? 256 : (NR == 2 ? 384 : (sizeof(S) == 8 && !DOTS ? 640 : 512));
+  return stencil_threads((int)sizeof(S), NR, DOTS);
 }
 
 template <typename S, typename G, int NL, int NT, int NR, bool DOTS, bool WIDE>
@@ -557,6 +549,10 @@ static int launch_mr_t(const DslashCall& d, const MrFuseArgs& F, cudaStream_t st
 template <typename S, typename G, int NL, int NT, int NR, bool WIDE = false>
 static int launch_nt(const WilsonArgs<S, G, NL>& A, int nrhs, cudaStream_t st) {
   dim3 grid((A.V + NT - 1) / NT, nrhs / NR);
+  // FP64 is bound by its arithmetic: a CTA more on one SM costs what the others do (8^3 x 16, 4 right-hand sides, 256
+  // CTAs: 67 us, crowded 99)
+  const ChainOff crowded(sizeof(S) == 16 &&
+                         !chain_fits((long)grid.x * grid.y, wilson_threads<S, NR, false>() / NT, sm_count()));
   if (A.z) {
     if constexpr (NT == 128) {  // the only CTA size of the dots (kShapesDots)
       const int k = dot_tiles(grid.x, nrhs, wilson_threads<S, 1, true>() / NT, sizeof(S));

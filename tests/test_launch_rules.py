@@ -1,6 +1,8 @@
 """The launch rules (csrc/launch_rules.h, plain C++) over the sizes that hierarchies have, compiled for the host.
 
-- coarse stencil: every tile it picks has a kernel, fits the reduction's partials, and leaves few lanes idle.
+- coarse stencil: every tile it picks has a kernel, fits the reduction's partials, and leaves few lanes idle;
+- fine stencil: the FP64 kernel needs 144 registers, and a larger budget only makes more waves;
+- early starts: launches that would crowd their predecessor wait for its end.
 """
 import os
 import shutil
@@ -45,3 +47,16 @@ def test_coarse_tiles(tmp_path):
         # lanes: FP64 (bound by arithmetic) idles in the last CTA alone, the others less than a third of a row
         assert pitch == groups if elem == 16 else 2 * pitch < 3 * groups, case
         assert pitch == groups or pitch % lb == 0, case
+
+
+def test_fp64_stencil_budget(tmp_path):
+    (threads,), = _run(tmp_path, 'printf("%d\\n", stencil_threads(16, 1, false));')
+    assert 65536 // threads // 8 * 8 < 144 + 32
+
+
+def test_crowded_launches_wait(tmp_path):
+    # CTAs, places of an SM, whether an early start pays (FP64 transfers, even-odd split, FP64 stencils, measured)
+    cases = [(384, 6, 1), (512, 6, 0), (625, 6, 0), (768, 6, 1), (324, 5, 1), (432, 5, 0), (648, 5, 1), (256, 3, 0),
+             (336, 3, 0), (1024, 3, 1)]
+    rows = _run(tmp_path, "\n".join('printf("%%d\\n", (int)chain_fits(%d, %d, 152));' % c[:2] for c in cases))
+    assert [r[0] for r in rows] == [c[2] for c in cases]
