@@ -663,6 +663,11 @@ int vcycle(mg_handle* h, int l, const void* r, void* e, int nrhs) {
   const Agg g = agg_of(a);
   const double pbytes = (double)a.Vc * 2 * a.nv * a.nhalf * a.bsites * bytes_of(prec);  // P once
   const double fbytes = (double)a.n() * bytes_of(prec) * nrhs, cbytes = (double)h->lev[l + 1]->n() * bytes_of(pc) * nrhs;
+  // FP64 transfers above 2 us wait for their predecessor's end.  Started early they leave the SMs at different times, the
+  // stencil behind them (one wave) piles up where room comes first, and each launch of the smoother inherits that
+  // placement: a V-cycle on 8^3 x 16, nv = 8: 280 us, 439 with both started early (12^4: 492 and 527).  Smaller ones
+  // gain: 4^4, three levels, 597 us against 615.
+  const bool long64 = prec == MG_F64 && 8.0 * a.nv * a.n() * nrhs > 2.5e6;
   const bool xmma = (prec == MG_F16 || prec == MG_BF16) && transfer_mma_ok(g, nrhs);
   int rvar = -1, pvar = -1;
   if (xmma) {
@@ -681,6 +686,7 @@ int vcycle(mg_handle* h, int l, const void* r, void* e, int nrhs) {
   }
   {
     Prof pf(h, MG_K_RESTRICT, prec, pbytes + fbytes + cbytes);
+    const ChainOff even(long64);
     LK(launch_restrict(prec, prec, pc, g, a.P[prec].p, res, rc, nrhs, h->st, rvar));
   }
   if (l + 1 == L - 1) {
@@ -703,6 +709,7 @@ int vcycle(mg_handle* h, int l, const void* r, void* e, int nrhs) {
   }
   {
     Prof pf(h, MG_K_PROLONG, prec, pbytes + fbytes + cbytes);
+    const ChainOff even(long64);
     LK(launch_prolong(pc, prec, prec, g, a.P[prec].p, ec, xc, nrhs, h->st, pvar));
   }
   // alpha = <A x_c|r0> / <A x_c|A x_c>  (Eq. 3.5);  e += alpha x_c, r0 -= alpha A x_c

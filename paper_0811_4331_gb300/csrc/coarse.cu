@@ -341,6 +341,9 @@ __global__ void __launch_bounds__(NT) prolong_kernel(const Agg g, const SP* P, c
   }
 }
 
+// FP64 transfers are bound by their arithmetic, so an SM with one CTA more than the others sets their time: they start
+// early only where they fit (launch_rules.h; 512 aggregates of 2^4, nv = 32, prolongation: 29 us, crowded 38.7; with nv = 4 the
+// early start is worth more, 6.4 us against 8.1).
 template <typename SI, typename SP, typename SO>
 static int restrict_t(const Agg& g, const void* P, const void* in, void* out, int nrhs, cudaStream_t st) {
   typedef typename Store<SP>::R R;
@@ -350,7 +353,12 @@ static int restrict_t(const Agg& g, const void* P, const void* in, void* out, in
   if (sm > 48 * 1024)
     allow_big_smem(restrict_kernel<SI, SP, SO, NT>);
   const int ngroups = (2 * g.nv + NT / 32 - 1) / (NT / 32);
-  launch_chain(restrict_kernel<SI, SP, SO, NT>, dim3(g.Vc * ngroups, nrhs), NT, sm, st, g, (const SP*)P, (const SI*)in, (SO*)out);
+  const dim3 grid(g.Vc * ngroups, nrhs);
+  static std::atomic<unsigned long long> held{0};
+  const ChainOff crowded(sizeof(R) == 8 && !chain_fits((long)grid.x * grid.y, ctas_held(held, restrict_kernel<SI, SP, SO, NT>, NT, sm),
+                                                       sm_count()));
+  launch_chain(restrict_kernel<SI, SP, SO, NT>, grid, NT, sm, st, g,
+               (const SP*)P, (const SI*)in, (SO*)out);
   return launched() ? 0 : -1;
 }
 
@@ -360,7 +368,12 @@ static int prolong_t(const Agg& g, const void* P, const void* in, void* out, int
   constexpr int NT = 256;
   const size_t sm = (size_t)2 * g.nv * sizeof(cx<R>);
   const int ngroups = (g.ncomp * g.bsites + NT - 1) / NT;
-  launch_chain(prolong_kernel<SI, SP, SO, NT>, dim3(g.Vc * ngroups, nrhs), NT, sm, st, g, (const SP*)P, (const SI*)in, (SO*)out);
+  const dim3 grid(g.Vc * ngroups, nrhs);
+  static std::atomic<unsigned long long> held{0};
+  const ChainOff crowded(sizeof(R) == 8 && g.nv >= 8 && !chain_fits((long)grid.x * grid.y, ctas_held(held, prolong_kernel<SI, SP, SO, NT>, NT, sm),
+                                                       sm_count()));
+  launch_chain(prolong_kernel<SI, SP, SO, NT>, grid, NT, sm, st, g,
+               (const SP*)P, (const SI*)in, (SO*)out);
   return launched() ? 0 : -1;
 }
 

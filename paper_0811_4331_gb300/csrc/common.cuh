@@ -7,6 +7,7 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <utility>
 
 namespace wmg {
@@ -90,6 +91,15 @@ inline int ctas_per_sm(K kern, int threads, size_t smem) {
     cudaGetLastError();
     n = 0;
   }
+  return n;
+}
+// The same through a word that keeps the last answer: shared memory in the upper bits, CTAs + 1 in the low byte.
+template <typename K>
+inline int ctas_held(std::atomic<unsigned long long>& last, K kern, int threads, size_t smem) {
+  const unsigned long long v = last.load(std::memory_order_relaxed);
+  if ((v & 255) && v >> 8 == smem) return (int)(v & 255) - 1;
+  const int n = ctas_per_sm(kern, threads, smem);
+  last.store((unsigned long long)smem << 8 | (unsigned)(n + 1), std::memory_order_relaxed);
   return n;
 }
 template <typename... P, typename... A>

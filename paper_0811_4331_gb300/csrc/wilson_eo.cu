@@ -248,6 +248,9 @@ static int split_t(const void* full, void* even, void* odd, const int L[4], size
                    cudaStream_t st) {
   const int Vh = L[0] * L[1] * L[2] * L[3] / 2;
   dim3 grid((Vh + 255) / 256, (unsigned)rows);
+  // FP64 chunks move enough for a crowded launch (chain_fits) to cost more than its early start gives: 11.0 us, 10.3 plain
+  static const int per_sm = sizeof(T) == 64 ? ctas_per_sm(eo_split_kernel<T>, 256, 0) : 0;
+  const ChainOff crowded(per_sm && !chain_fits((long)grid.x * grid.y, per_sm, sm_count()));
   launch_chain(eo_split_kernel<T>, grid, 256, 0, st, (const T*)full, (T*)even, (T*)odd, L[0], L[1], L[2], Vh, hstride);
   return launched() ? 0 : -1;
 }
