@@ -443,18 +443,25 @@ int launch_coarse_mma(int prec, const void* Cf, const void* in, void* out, const
   const int npad = (n + 15) / 16 * 16, T = npad / 16;
   const int V = L[0] * L[1] * L[2] * L[3];
   const int NT8all = (R + 7) / 8;
-  int NT8 = NT8all;  // default: one CTA per coarse site holds every right-hand side
+  int NT8 = NT8all;  // default: one CTA per coarse site holds every right-hand side, if they fit
   if (variant >= 0) {
     int seen = -1;
     for (int v = 0; v < kMmaVariants; ++v)
       if (kMmaTiles[v] <= NT8all && ++seen == variant) NT8 = kMmaTiles[v];
   }
-  const int splits = (NT8all + NT8 - 1) / NT8;
-  const size_t sm = (size_t)9 * NT8 * 8 * row_pitch(npad);
-  if ((size_t)9 * NT8 * 8 * 4 * npad > 200 * 1024 || T > 32) return -1;
+  if (T > 32) return -1;
   size_t stage = 0;
   const int ns = stream_stages(T, NT8, &stage);
   unsigned char* rows = coarse_mma_scratch_bytes(n, V, R) ? (unsigned char*)scratch : nullptr;
+  if (ns * stage + 2048 > (size_t)smem_optin_bytes()) rows = nullptr;
+  if (!rows) {  // the direct form holds the nine directions: as many tiles as fit, in even groups
+    const int most = (int)(200 * 1024 / ((size_t)9 * 8 * 4 * npad));
+    if (most < 1) return -1;
+    const int groups = (NT8all + most - 1) / most;
+    if (NT8 > most) NT8 = (NT8all + groups - 1) / groups;
+  }
+  const int splits = (NT8all + NT8 - 1) / NT8;
+  const size_t sm = (size_t)9 * NT8 * 8 * row_pitch(npad);
   if (rows) {
     const size_t smr = (size_t)32 * (4 * npad + 4);
     const dim3 g((unsigned)((V + 31) / 32), (unsigned)R);
