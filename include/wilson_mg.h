@@ -286,7 +286,13 @@ int schur_apply(mg_handle* h, int prec, const void* in, void* out, int nrhs, voi
  * (A_l = P^+ A_{l-1} P, Sec. 2), internal layout, device memory.
  * Precisions: the vector storage; the operator is held in the same
  * precision, except that with coarse_mma an FP32 call runs on tensor cores
- * with the operator in BF16 (FP32 accumulation).
+ * with the operator in BF16 (FP32 accumulation).  Four and more right-hand
+ * sides of that form are first rounded to BF16 in a buffer that the handle
+ * keeps for each stream (eight at most, until mg_release_work) and for each
+ * stream of each capture (sixteen at most, until mg_destroy); further ones use
+ * no memory of the handle but the operator, at a lower speed, with the same
+ * result.  So calls with different outputs on different streams are
+ * independent, and a captured call stays valid as long as the handle.
  * Errors: MG_EINVAL (no such level / precision). */
 int coarse_apply(mg_handle* h, int level, int prec, const void* in, void* out, int nrhs,
                  void* stream);

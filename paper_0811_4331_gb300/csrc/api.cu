@@ -129,6 +129,39 @@ void* work(mg_handle* h, int l, int prec, int idx, int nrhs, int count = 1) {
   return vecs[idx]->p;
 }
 
+// Rows for one coarse_apply on `st`.  Calls on other streams may overlap, and a graph captured by the caller is replayed
+// whenever it likes, so neither shares a buffer with anything else.  Null (the stencil gathers its vectors itself, the
+// same bits) where there is no memory, and on further streams and captures than kRowStreams and kRowCaptures.
+constexpr size_t kRowStreams = 8, kRowCaptures = 16;
+void* call_rows(mg_handle* h, cudaStream_t st, size_t bytes, bool* captured) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  unsigned long long id = 0, seq = 0;
+  if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap == cudaStreamCaptureStatusInvalidated) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  *captured = cap == cudaStreamCaptureStatusActive;
+  // (a capturing stream has no id to ask for, but its handle is its own while it captures)
+  if ((*captured ? cudaStreamGetCaptureInfo(st, &cap, &seq) : cudaStreamGetId(st, &id)) != cudaSuccess ||
+      (*captured && seq == 0)) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  if (*captured) id = (unsigned long long)(uintptr_t)st;
+  size_t like = 0;
+  for (auto& r : h->call_rows) {
+    like += (r->capture != 0) == *captured;
+    if (r->stream != id || r->capture != seq) continue;
+    if (bytes <= r->buf.bytes) return r->buf.p;
+    if (!*captured) return r->buf.ensure(bytes) ? r->buf.p : nullptr;
+  }
+  if (like >= (*captured ? kRowCaptures : kRowStreams)) return nullptr;
+  std::unique_ptr<mg_handle::StreamRows> r(new mg_handle::StreamRows{id, seq, {}});
+  if (!(*captured ? r->buf.take(bytes) : r->buf.ensure(bytes))) return nullptr;
+  h->call_rows.push_back(std::move(r));
+  return h->call_rows.back()->buf.p;
+}
+
 int ensure_reducer(mg_handle* h, int nrhs) {
   if (nrhs > kMaxRhs) {
     set_error("nrhs above the library limit of 64");
@@ -216,6 +249,11 @@ int tuned(mg_handle* h, K&& key_of, int nvar, F&& run) {
   auto it = g_tune.find(key);
   if (it != g_tune.end()) return it->second.variant;
   if (h->capturing) return -1;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(h->st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+    cudaGetLastError();
+    return -1;  // nothing can be timed inside a caller's capture
+  }
   cudaEvent_t e0, e1;
   if (cudaEventCreate(&e0) != cudaSuccess) return -1;
   if (cudaEventCreate(&e1) != cudaSuccess) {
@@ -257,9 +295,10 @@ std::string tkey(const char* kernel, std::initializer_list<long long> v) {
   return k;
 }
 
-// out = a_ * (A_l in) + c_ * y; optional dots <out|z>, ||out||^2 into slot.
+// out = a_ * (A_l in) + c_ * y; optional dots <out|z>, ||out||^2 into slot.  `alone`: a call of its own (coarse_apply),
+// which shares no scratch with the handle's solves or its other calls.
 int op_apply(mg_handle* h, int l, int prec, const void* in, void* out, const void* y, double a_, double c_,
-             const void* z, size_t slot, int nrhs) {
+             const void* z, size_t slot, int nrhs, bool alone = false) {
   Level& a = *h->lev[l];
   if (l == 0) {
     if (!a.links[prec].p) {
@@ -301,22 +340,29 @@ int op_apply(mg_handle* h, int l, int prec, const void* in, void* out, const voi
     // tensor cores: out = a_ A in + c_ y, then the dots in a separate deterministic pass
     const double vb = (double)a.n() * bytes_of(prec);
     void* rows = nullptr;  // the vectors' BF16 rows
+    bool captured = false;
     if (const size_t rb = coarse_mma_scratch_bytes(a.ncomp, a.V, nrhs)) {
-      rows = work(h, l, prec, WV_ROWS, nrhs, (int)((rb + (size_t)vb * nrhs - 1) / ((size_t)vb * nrhs)));
-      if (!rows) {
-        set_error("no work buffer for the coarse stencil's rows");
-        return MG_ENOMEM;
+      if (alone) {
+        rows = call_rows(h, h->st, rb, &captured);
+      } else {
+        rows = work(h, l, prec, WV_ROWS, nrhs, (int)((rb + (size_t)vb * nrhs - 1) / ((size_t)vb * nrhs)));
+        if (!rows) {
+          set_error("no work buffer for the coarse stencil's rows");
+          return MG_ENOMEM;
+        }
       }
     }
     {
       DevBuf scratch;
-      const int var = tuned(h, [&] { return tkey("coarse_mma", {prec, a.ncomp, a.V, nrhs}); }, coarse_mma_variants(nrhs), [&](int v) {
+      const int var = tuned(h, [&] { return tkey(rows ? "coarse_mma" : "coarse_mma_direct", {prec, a.ncomp, a.V, nrhs}); }, coarse_mma_variants(nrhs), [&](int v) {
         if (!scratch.p && !scratch.ensure((size_t)vb * nrhs)) return -1;
         return launch_coarse_mma(prec, a.cop_mma.p, in, scratch.p, y, a.L, a.ncomp, nrhs, a_, c_, h->st, v, mmshift,
                                  rows);
       });
       Prof pf(h, MG_K_COARSE, MG_BF16, (double)mma_pack_bytes(a.ncomp, a.V) + nrhs * vb * (2 + (y != nullptr)));
       if (rows) count_launches(1);
+      // in a graph the two launches start early at a loss (512 sites, n = 48, 24 right-hand sides: 18.8 us, 15.5 plain)
+      const ChainOff plain(captured && rows);
       LK(launch_coarse_mma(prec, a.cop_mma.p, in, out, y, a.L, a.ncomp, nrhs, a_, c_, h->st, var, mmshift, rows));
     }
     if (z) {
@@ -892,7 +938,6 @@ size_t mg_release_work(mg_handle* h, void* stream) {
     cudaGetLastError();
     return 0;  // work may still be queued on the buffers: keep them
   }
-  DevIdleScope idle;  // both streams the handle's solves use are done
   size_t freed = 0;
   auto drop = [&](DevBuf& d) {
     if (d.p) {
@@ -900,6 +945,11 @@ size_t mg_release_work(mg_handle* h, void* stream) {
       d.release();
     }
   };
+  auto& rows = h->call_rows;  // of any stream; those of captures stay for the graphs that use them
+  for (auto& r : rows)
+    if (!r->capture) drop(r->buf);
+  rows.erase(std::remove_if(rows.begin(), rows.end(), [](const auto& r) { return !r->capture; }), rows.end());
+  DevIdleScope idle;  // both streams the handle's solves use are done
   for (auto& byprec : h->work)
     for (auto& vecs : byprec)
       for (auto& v : vecs)
@@ -932,6 +982,7 @@ size_t mg_handle_bytes(const mg_handle* h) {
     for (const auto& vecs : byprec)
       for (const auto& v : vecs)
         if (v) add(*v);
+  for (const auto& r : h->call_rows) add(r->buf);
   add(h->red.partials);
   add(h->red.tickets);
   add(h->red.slots);
@@ -1668,7 +1719,7 @@ int coarse_apply(mg_handle* h, int level, int prec, const void* in, void* out, i
   cudaStream_t keep = h->st;
   h->st = (cudaStream_t)stream;
   int rc = ensure_reducer(h, nrhs);
-  if (rc == MG_OK) rc = op_apply(h, level, prec, in, out, nullptr, 1.0, 0.0, nullptr, 0, nrhs);
+  if (rc == MG_OK) rc = op_apply(h, level, prec, in, out, nullptr, 1.0, 0.0, nullptr, 0, nrhs, true);
   h->st = keep;
   return rc;
 }

@@ -163,6 +163,21 @@ struct DevBuf {
     bytes = c;
     return true;
   }
+  // A first allocation of n bytes that neither synchronises nor frees (permitted while this thread captures).
+  bool take(size_t n) {
+    const size_t c = DevCache::size_class(n);
+    p = dev_cache().take(c);
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;  // cudaMalloc is not part of what is captured
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (!p && cudaMalloc(&p, c) != cudaSuccess) {
+      cudaGetLastError();
+      p = nullptr;
+    }
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (p) g_dev_allocs.fetch_add(1, std::memory_order_relaxed);
+    bytes = p ? c : 0;
+    return p != nullptr;
+  }
   template <typename T>
   T* as() const {
     return (T*)p;
@@ -238,6 +253,14 @@ struct mg_handle {
   // work vectors: [level][precision][index]
   std::vector<std::vector<std::vector<std::unique_ptr<wmg::DevBuf>>>> work;
   int work_nrhs = 0;
+  // BF16 rows of coarse_apply: a buffer for each of the first streams it is called on (a stream's id is its own for the
+  // life of the program, so a buffer is only ever reused in stream order), and for each of the first streams and stream
+  // captures it is captured in (capture: the sequence's id, else 0), which the captured graph keeps using
+  struct StreamRows {
+    unsigned long long stream, capture;
+    wmg::DevBuf buf;
+  };
+  std::vector<std::unique_ptr<StreamRows>> call_rows;
   // outer solver buffers
   wmg::DevBuf gr, gW, gZ, gb64, gx64, gr64, gtmp;
   wmg::DevBuf gH, galpha, gy;  // outer GCR: H (A Z = W H), alpha, y = H^-1 alpha per right-hand side
