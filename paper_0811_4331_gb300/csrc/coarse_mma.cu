@@ -300,10 +300,9 @@ __device__ __forceinline__ void bulk_copy(unsigned dst, const void* src, unsigne
                "l"(src), "r"(bytes), "r"(bar)
                : "memory");
 }
-// Bounded wait for the phase of the given parity; false when it ran out.
-constexpr int kSpinMax = 1 << 18;
-__device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity) {
-  for (int i = 0; i < kSpinMax; ++i) {
+// Wait for the phase of the given parity, at most `spins` tries; false when they ran out.
+__device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity, int spins) {
+  for (int i = 0; i < spins; ++i) {
     unsigned ok;
     asm volatile(
         "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
@@ -321,7 +320,7 @@ template <typename S, int NT8>
 __global__ void __launch_bounds__(224)
     coarse_stream_kernel(const unsigned char* Cf, const S* in, const unsigned char* rows, S* out, const S* y2, int L0,
                          int L1, int L2, int L3, int n, int npad, int R, float a, float c, const double* shift,
-                         int splits, int items, int ns) {
+                         int splits, int items, int ns, int spins) {
   chain_begin();
   extern __shared__ __align__(128) unsigned char smem_ring[];
   __shared__ __align__(8) unsigned long long bars[2 * kMaxStages];  // full, empty
@@ -353,7 +352,7 @@ __global__ void __launch_bounds__(224)
       const unsigned rbytes = Rc * pitch;
 #pragma unroll
       for (int d = 0; d < 9; ++d) {
-        ok = ok && mbar_wait(empty + 8 * slot, ph ^ 1u);
+        ok = ok && mbar_wait(empty + 8 * slot, ph ^ 1u, spins);
         if (!ok) break;
         const unsigned bar = full + 8 * slot, dst = ring + slot * stage;
         mbar_expect(bar, abytes + rbytes);
@@ -371,7 +370,7 @@ __global__ void __launch_bounds__(224)
       for (int i = 0; i < (issued < ns ? issued : ns); ++i) {
         slot = slot == 0 ? ns - 1 : slot - 1;
         if (slot == ns - 1) ph ^= 1u;
-        mbar_wait(full + 8 * slot, ph);
+        mbar_wait(full + 8 * slot, ph, spins);
       }
     return;
   }
@@ -382,8 +381,10 @@ __global__ void __launch_bounds__(224)
     const int B = w / splits, r0 = (w - B * splits) * NT8 * 8;
     float accr[NT8][4], acci[NT8][4];
     mma_zero<NT8>(accr, acci);
-    for (int d = 0; d < 9; ++d) {
-      ok = ok && mbar_wait(full + 8 * slot, ph);
+    for (int d = 0; d < 9 && ok; ++d) {
+      // a warp whose wait runs out reads and arrives no more: the others' stages stay theirs until their waits run out too
+      ok = __all_sync(0xffffffffu, mbar_wait(full + 8 * slot, ph, spins));
+      if (!ok) break;
       unsigned ya = ya0 + slot * stage;
       const unsigned char* af = af0 + (size_t)slot * stage;
 #pragma unroll 3
@@ -400,7 +401,12 @@ __global__ void __launch_bounds__(224)
         ph ^= 1u;
       }
     }
-    if (!ok) accr[0][0] = accr[0][1] = accr[0][2] = accr[0][3] = __int_as_float(0x7fc00000);  // the solver refuses NaN
+    if (!ok) {  // every output of this item and the next ones: the solver refuses NaN
+#pragma unroll
+      for (int q = 0; q < NT8; ++q)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) accr[q][k] = acci[q][k] = __int_as_float(0x7fc00000);
+    }
     mma_store<S, NT8>(accr, acci, in, out, y2, shift, B, V, warp, r0, n, R, a, c);
   }
 }
@@ -438,7 +444,7 @@ int coarse_mma_variants(int R) {
 }
 
 int launch_coarse_mma(int prec, const void* Cf, const void* in, void* out, const void* y2, const int L[4], int n, int R,
-                      double a, double c, cudaStream_t st, int variant, const double* shift, void* scratch) {
+                      double a, double c, cudaStream_t st, int variant, const double* shift, void* scratch, int spins) {
   if (prec != 1 && prec != 3) return -1;
   const int npad = (n + 15) / 16 * 16, T = npad / 16;
   const int V = L[0] * L[1] * L[2] * L[3];
@@ -481,7 +487,7 @@ int launch_coarse_mma(int prec, const void* Cf, const void* in, void* out, const
     auto kern = coarse_stream_kernel<S, K>;                                                                 \
     allow_big_smem(kern);                                                                                   \
     launch_chain(kern, ctas, 32 * (T + 1), ring, st, (const unsigned char*)Cf, (const S*)in, rows, (S*)out, (const S*)y2, L[0], \
-                                           L[1], L[2], L[3], n, npad, R, (float)a, (float)c, shift, splits, items, ns); \
+                                           L[1], L[2], L[3], n, npad, R, (float)a, (float)c, shift, splits, items, ns, spins); \
   } else {                                                                                                  \
     auto kern = coarse_mma_kernel<S, K>;                                                                    \
     if (sm > 40 * 1024) allow_big_smem(kern);                                                               \

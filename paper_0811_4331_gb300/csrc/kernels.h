@@ -195,7 +195,8 @@ int launch_mma_pack(const double2* C, int n, int V, void* out, cudaStream_t st);
 // sides split over CTAs); every shape gives bit-identical results.
 int launch_coarse_mma(int prec, const void* Cf, const void* in, void* out, const void* y2, const int L[4], int n, int R,
                       double a, double c, cudaStream_t st, int variant = -1, const double* shift = nullptr,
-                      void* scratch = nullptr);
+                      void* scratch = nullptr, int spins = 1 << 18);
+// spins: tries of a wait between the streaming form's copies and its products; outputs whose wait runs out are NaN.
 // scratch: coarse_mma_scratch_bytes (0 for few right-hand sides); without it every CTA gathers its vectors itself,
 // with the same result.
 size_t coarse_mma_scratch_bytes(int n, int V, int R);
