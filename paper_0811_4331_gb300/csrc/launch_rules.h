@@ -2,6 +2,7 @@
 // given sizes takes.  Plain C++ (no CUDA), so that they can be checked on any
 // host.
 #pragma once
+#include <limits.h>
 #include <stddef.h>
 
 namespace wmg {
@@ -111,6 +112,39 @@ inline CoarseShape coarse_shape(size_t elem, long n, long V, int nrhs, int sms) 
 //   pipe, 16^3 x 32 takes 233 with either
 constexpr int stencil_threads(int elem, int nr, bool dots) {
   return elem == 16 ? 384 : (nr == 2 ? 384 : (elem == 8 && !dots ? 640 : 512));
+}
+
+// Tiles of 128 sites per CTA of a launch with fused dots: `lanes` rows of `tiles`
+// tiles (a row is one or two right-hand sides), `per_sm` CTAs on an SM.  Each tile
+// keeps its own partial sums, so the result does not depend on the choice.
+//
+// FP32: a CTA's start and its last reduction step take about 0.3 tile times
+// whatever its tiles, and a wave as long as its longest CTA: the largest number
+// within 3 % of the shortest waves, at most 24, or 32 in a single wave.  16 x 8 x
+// 8 x 16, 64 right-hand sides: 88 us (one tile per CTA 109, fourteen, which are
+// 640 CTAs on 608 places, 123); 24^4, 24 right-hand sides: one tile 792, eighteen
+// 658; 16^3 x 32, 12, two right-hand sides per thread: 184 -> 129 with its own
+// lanes and places instead of those of one per thread.
+// 16 bits, where a tile is longer: one below eight waves, else about four, in
+// whole waves on average (16^3 x 32, FP16, 12: 134 with one tile, 127; the rule
+// above 124, but 112 instead of 108 on 12^4 with 64).
+inline int dot_tiles(long tiles, long lanes, int per_sm, int sms, int elem) {
+  const long total = tiles * lanes, places = (long)per_sm * sms;
+  if (elem != 8) {
+    if (total < places * 8) return 1;
+    const long waves = total / (places * 4);
+    return (int)((total + places * waves - 1) / (places * waves));
+  }
+  auto time = [&](int k) {
+    const long waves = ((tiles + k - 1) / k * lanes + places - 1) / places;
+    return k > 24 && waves > 1 ? LONG_MAX / 100 : waves * (10 * k + 3);
+  };
+  const int most = 32;
+  long least = time(1);
+  for (int k = 2; k <= most; ++k) least = time(k) < least ? time(k) : least;
+  int best = most;
+  while (100 * time(best) > 103 * least) --best;
+  return best;
 }
 
 // ------------------------------------------------------------------ chained launches

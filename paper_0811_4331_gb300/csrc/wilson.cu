@@ -495,22 +495,6 @@ __global__ void __launch_bounds__(256) wilson_small_mr_kernel(const WilsonArgs<S
   grid_reduce<3, 256, R>(red, A.red, rhs);
 }
 
-// Tiles per CTA of a launch with fused dots, of which an SM holds `per_sm` CTAs:
-// CTAs of at most about 16 (FP32) or 4 (16-bit) tiles that fill whole waves, so
-// that few tiles pay for a reduction and none waits for a nearly empty last
-// wave; one tile where 16-bit launches have less than eight waves.  Each tile
-// keeps its own partial sums, so the result does not depend on the choice.
-// 16^3 x 32, 12 right-hand sides, one tile per CTA -> this: FP16 134 -> 129 us,
-// FP32 181 -> 155 (one partial per CTA instead: 124 and 148, but the null
-// vectors' last bits moved, and with them 16-bit roundings of P).
-static int dot_tiles(unsigned tiles, int nrhs, int per_sm, size_t elem) {
-  const size_t total = (size_t)tiles * nrhs, slots = (size_t)per_sm * sm_count();
-  size_t waves = total / (slots * (elem == 8 ? 16 : 4));
-  if (elem != 8 && total < slots * 8) return 1;
-  waves = waves < 1 ? 1 : waves;
-  return (int)((total + slots * waves - 1) / (slots * waves));
-}
-
 template <typename S, typename G, int NL>
 static int launch_mr_t(const DslashCall& d, const MrFuseArgs& F, cudaStream_t st) {
   WilsonArgs<S, G, NL> A;
@@ -536,7 +520,7 @@ static int launch_mr_t(const DslashCall& d, const MrFuseArgs& F, cudaStream_t st
     }
     constexpr int NT = 128;
     const unsigned tiles = (unsigned)((A.V + NT - 1) / NT);
-    const int k = dot_tiles(tiles, d.nrhs, kMrThreads / NT, sizeof(S));
+    const int k = dot_tiles(tiles, d.nrhs, kMrThreads / NT, sm_count(), (int)sizeof(S));
     const dim3 grid((tiles + k - 1) / k, d.nrhs);
     if ((((uintptr_t)d.in | (uintptr_t)F.pprev) & 31u) == 0)
       wilson_mr_tiles_kernel<S, G, NL, NT, true><<<grid, NT, 0, st>>>(A, F);
@@ -555,7 +539,7 @@ static int launch_nt(const WilsonArgs<S, G, NL>& A, int nrhs, cudaStream_t st) {
                          !chain_fits((long)grid.x * grid.y, wilson_threads<S, NR, false>() / NT, sm_count()));
   if (A.z) {
     if constexpr (NT == 128) {  // the only CTA size of the dots (kShapesDots)
-      const int k = dot_tiles(grid.x, nrhs, wilson_threads<S, 1, true>() / NT, sizeof(S));
+      const int k = dot_tiles(grid.x, nrhs / NR, wilson_threads<S, NR, true>() / NT, sm_count(), (int)sizeof(S));
       grid.x = (grid.x + k - 1) / k;
       launch_chain(wilson_kernel<S, G, NL, NT, NR, true, WIDE>, grid, NT, 0, st, A);
     } else {

@@ -60,3 +60,21 @@ def test_crowded_launches_wait(tmp_path):
              (336, 3, 0), (1024, 3, 1)]
     rows = _run(tmp_path, "\n".join('printf("%%d\\n", (int)chain_fits(%d, %d, 152));' % c[:2] for c in cases))
     assert [r[0] for r in rows] == [c[2] for c in cases]
+
+
+def test_dot_tiles_fill_their_waves(tmp_path):
+    """FP32: waves times tiles per CTA, with a CTA's own 0.3 tile times, within 3 % of the best of the range; and two
+    right-hand sides per thread count their own rows and places."""
+    rows = _run(tmp_path, """
+  for (long tiles = 9; tiles < 20000; tiles += tiles / 5 + 1)
+    for (long lanes = 1; lanes <= 64; lanes += lanes < 8 ? 1 : 8)
+      for (int per_sm = 3; per_sm <= 4; ++per_sm)
+        printf("%ld %ld %d %d\\n", tiles, lanes, per_sm, dot_tiles(tiles, lanes, per_sm, 152, 8));""")
+    for tiles, lanes, per_sm, k in rows:
+        def time(q):
+            waves = -(-(-(-tiles // q) * lanes) // (per_sm * 152))
+            return float("inf") if q > 24 and waves > 1 else waves * (q + 0.3)
+
+        assert 1 <= k <= 32 and time(k) <= 1.031 * min(time(q) for q in range(1, 33)), (tiles, lanes, per_sm)
+    src = open(os.path.join(CSRC, "wilson.cu")).read()
+    assert "dot_tiles(grid.x, nrhs / NR, wilson_threads<S, NR, true>() / NT" in src
