@@ -719,12 +719,12 @@ int vcycle(mg_handle* h, int l, const void* r, void* e, int nrhs) {
   if (xmma) {
     DevBuf scratch;
     const size_t need = (size_t)std::max(fbytes, cbytes);
-    rvar = tuned(h, [&] { return tkey("restrict_mma", {prec, pc, a.nv, a.bsites, a.Vc, nrhs}); }, transfer_mma_variants(g, nrhs, false),
+    rvar = tuned(h, [&] { return tkey("restrict_mma", {prec, pc, a.nv, a.bsites, a.Vc, nrhs}); }, transfer_mma_variants(g, nrhs, false, pc),
                  [&](int v) {
                    if (!scratch.p && !scratch.ensure(need)) return -1;
                    return launch_restrict(prec, prec, pc, g, a.P[prec].p, res, scratch.p, nrhs, h->st, v);
                  });
-    pvar = tuned(h, [&] { return tkey("prolong_mma", {prec, pc, a.nv, a.bsites, a.Vc, nrhs}); }, transfer_mma_variants(g, nrhs, true),
+    pvar = tuned(h, [&] { return tkey("prolong_mma", {prec, pc, a.nv, a.bsites, a.Vc, nrhs}); }, transfer_mma_variants(g, nrhs, true, pc),
                  [&](int v) {
                    if (!scratch.p && !scratch.ensure(need)) return -1;
                    return launch_prolong(pc, prec, prec, g, a.P[prec].p, rc, scratch.p, nrhs, h->st, v);

@@ -227,7 +227,7 @@ int launch_restrict_mma(int pin, int pP, int pout, const Agg& g, const void* P, 
 int launch_prolong_mma(int pin, int pP, int pout, const Agg& g, const void* P, const void* in, void* out, int nrhs,
                        cudaStream_t st, int variant = -1);
 // Launch shapes of the tensor-core transfers (work split over CTAs; bit-identical results).
-int transfer_mma_variants(const Agg& g, int nrhs, bool prolong);
+int transfer_mma_variants(const Agg& g, int nrhs, bool prolong, int coarse_prec);
 
 // C_0(B) += delta 1 on a coarse stencil [9][n][n][V] (FP64).
 int launch_diag_shift(double2* C, int n, int V, double delta, cudaStream_t st);

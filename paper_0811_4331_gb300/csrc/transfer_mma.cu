@@ -711,8 +711,8 @@ static const int kRTiles[] = {2, 1};
 static const PTile kPTiles[] = {{1, 3}, {2, 2}, {4, 2}, {16, 2}};
 constexpr int kRShapes = 2, kPShapes = 4;
 
-int transfer_mma_variants(const Agg& g, int nrhs, bool prolong) {
-  if (tile_geom(g)) return (prolong ? kPShapes : kRShapes) * (nrhs > 16 ? 2 : 1);
+int transfer_mma_variants(const Agg& g, int nrhs, bool prolong, int coarse_prec) {
+  if (tile_geom(g) && cx_bytes(coarse_prec) == 8) return (prolong ? kPShapes : kRShapes) * (nrhs > 16 ? 2 : 1);
   const int NT8 = (nrhs + 7) / 8;
   int nv = 0;
   for (int v = 0; v < kXVariants; ++v) nv += kXTiles[v] <= NT8 ? 1 : 0;
