@@ -1132,47 +1132,49 @@ __global__ void __launch_bounds__(kMmThreads)
 
 // Scratch of the tiled product: partial tiles (up to 8 K ranges x 64 rhs x N
 // complex FP64) and one ticket per 16-row tile.
+// A launch of about two CTAs per SM, bound by arithmetic: an SM with three would set its time (N = 2048, FP64, 24
+// right-hand sides: 2344 us, crowded 3588).
+template <typename K, typename... A>
+static void matmul_go(K kern, dim3 grid, cudaStream_t st, A... args) {
+  static const int per_sm = ctas_per_sm(kern, kMmThreads, 0);
+  const ChainOff crowded(!chain_fits((long)grid.x * grid.y, per_sm, sm_count()));
+  launch_chain(kern, grid, kMmThreads, 0, st, args...);
+}
+
 size_t dense_matvec_scratch_bytes(int N) {
   return (size_t)8 * 64 * N * 16 + (size_t)((N + kMmRows - 1) / kMmRows) * sizeof(unsigned) + 256;
 }
 
-// y = inv x (+ y if acc) for a few right-hand sides, or with a matrix per
-// right-hand side (midx, RB = 1).  CTA = kMvRows rows (two warps each, halves of
-// the columns) and RB right-hand sides, whose vectors it first stages in the
-// matrix's precision: a conversion from FP64 runs on the scarce FP64 pipe, and
-// one per row and column was half of the time.  The matrix is read in 16-byte
-// pieces, four in flight per lane; warp sums in a fixed order.
-// N = 1280, FP32 inverse, one right-hand side: 9.0 -> 6.1 us.
-constexpr int kMvRows = 4, kMvThreads = 64 * kMvRows;
+constexpr int kMvPiece = 2048;
 
-template <typename TM, typename SI, typename SO, int RB>
-__global__ void __launch_bounds__(kMvThreads) dense_matvec_kernel(int N, const TM* inv, const SI* x, SO* y, int nrhs,
-                                                                  int acc, const int* midx) {
+// y = inv x (+ y if acc), row form: CTA = ROWS rows (two warps each, halves of the
+// columns) of one right-hand side (with its own matrix if midx).  The vector is
+// staged first in the matrix's precision: a conversion from FP64 runs on the
+// scarce FP64 pipe, and one per row and column was half of the time.  PIECES
+// stages 2048 columns at a time, where all of them would leave an SM one or two
+// CTAs.  The matrix is read in 16-byte pieces, four in flight per lane; warp sums
+// in a fixed order.  Each right-hand side reads the matrix again, from L2 where it
+// fits: two or four of them per CTA took as long or longer (N = 1536, FP32, 4: 12
+// us alone, 17 together; FP64, 3: 58 and 85).
+// N = 1280, FP32 inverse, one right-hand side: 9.0 -> 6.1 us.  FP64, N = 8192, one:
+// 697 us with the whole vector staged, PIECES 456.
+template <typename TM, typename SI, typename SO, int ROWS, bool PIECES>
+__global__ void __launch_bounds__(64 * ROWS) dense_matvec_kernel(int N, const TM* inv, const SI* x, SO* y, int acc,
+                                                                 const int* midx) {
   chain_begin();
   typedef typename Store<TM>::R R;
   constexpr int E = (int)(16 / sizeof(TM));  // matrix elements per 16 bytes
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  cx<R>* xs = (cx<R>*)smem_raw;  // [RB][N]
-  __shared__ cx<R> part[kMvRows][2][RB];
-  const int r0 = blockIdx.y * RB, rows = min(RB, nrhs - r0);
-  for (int e = threadIdx.x; e < RB * N; e += kMvThreads) {
-    const int r = RB == 1 ? 0 : e / N;
-    xs[e] = r < rows ? ldc<R>(x, (size_t)r0 * N + e) : zero<R>();
-  }
-  __syncthreads();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, half = warp & 1;
-  const int row = blockIdx.x * kMvRows + (warp >> 1);
-  const int mid = (N / 2 + E - 1) / E * E, c0 = half ? mid : 0, c1 = half ? N : mid;
-  cx<R> a[RB];
-#pragma unroll
-  for (int r = 0; r < RB; ++r) a[r] = zero<R>();
-  if (row < N) {
-    const TM* rp = inv + (midx ? (size_t)midx[r0] * N * N : (size_t)0) + (size_t)row * N;
-    auto fma_col = [&](const cx<R>& m, int j) {
-#pragma unroll
-      for (int r = 0; r < RB; ++r) a[r] = cfma(m, xs[r * N + j], a[r]);
-    };
-    int j = c0;
+  cx<R>* xs = (cx<R>*)smem_raw;
+  __shared__ cx<R> part[ROWS][2];
+  const int r = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31, half = warp & 1;
+  const int row = blockIdx.x * ROWS + (warp >> 1);
+  const TM* rp0 = inv + (midx ? (size_t)midx[r] * N * N : (size_t)0) + (size_t)min(row, N - 1) * N;
+  cx<R> a = zero<R>();
+  auto columns = [&](int k0, int kn) {  // of the vector staged at xs
+    const int mid = (kn / 2 + E - 1) / E * E, c1 = half ? kn : mid;
+    const TM* rp = rp0 + k0;
+    int j = half ? mid : 0;
     if (E == 1 || N % E == 0) {  // rows start on 16 bytes
       auto load = [&](int at, cx<R> (&m)[E]) {
         if constexpr (E == 1) {
@@ -1190,26 +1192,36 @@ __global__ void __launch_bounds__(kMvThreads) dense_matvec_kernel(int N, const T
 #pragma unroll
         for (int u = 0; u < 4; ++u)
 #pragma unroll
-          for (int q = 0; q < E; ++q) fma_col(m[u][q], j + (u * 32 + lane) * E + q);
+          for (int q = 0; q < E; ++q) a = cfma(m[u][q], xs[j + (u * 32 + lane) * E + q], a);
       }
     }
-    for (j += lane; j < c1; j += 32) fma_col(ldc<R>(rp, j), j);
-  }
-#pragma unroll
-  for (int r = 0; r < RB; ++r) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      a[r].re += __shfl_down_sync(0xffffffffu, a[r].re, o);
-      a[r].im += __shfl_down_sync(0xffffffffu, a[r].im, o);
+    for (j += lane; j < c1; j += 32) a = cfma(ldc<R>(rp, j), xs[j], a);
+  };
+  if constexpr (PIECES) {
+    for (int k0 = 0; k0 < N; k0 += kMvPiece) {
+      const int kn = min(kMvPiece, N - k0);
+      if (k0 > 0) __syncthreads();  // the piece before is read
+      for (int e = threadIdx.x; e < kn; e += 64 * ROWS) xs[e] = ldc<R>(x, (size_t)r * N + k0 + e);
+      __syncthreads();
+      columns(k0, kn);
     }
-    if (lane == 0) part[warp >> 1][half][r] = a[r];
+  } else {
+    for (int e = threadIdx.x; e < N; e += 64 * ROWS) xs[e] = ldc<R>(x, (size_t)r * N + e);
+    __syncthreads();
+    if (row < N) columns(0, N);
   }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    a.re += __shfl_down_sync(0xffffffffu, a.re, o);
+    a.im += __shfl_down_sync(0xffffffffu, a.im, o);
+  }
+  if (lane == 0) part[warp >> 1][half] = a;
   __syncthreads();
-  if (threadIdx.x < kMvRows * RB) {
-    const int q = threadIdx.x % kMvRows, r = threadIdx.x / kMvRows, i = blockIdx.x * kMvRows + q;
-    if (i < N && r < rows) {
-      const cx<R> s = part[q][0][r] + part[q][1][r];
-      const size_t o = (size_t)(r0 + r) * N + i;
+  if (threadIdx.x < ROWS) {
+    const int q = threadIdx.x, i = blockIdx.x * ROWS + q;
+    if (i < N) {
+      const cx<R> s = part[q][0] + part[q][1];
+      const size_t o = (size_t)r * N + i;
       cx<double> v = mk<double>((double)s.re, (double)s.im);
       if (acc) v = v + ldc<double>(y, o);
       stc(y, o, v);
@@ -1217,39 +1229,35 @@ __global__ void __launch_bounds__(kMvThreads) dense_matvec_kernel(int N, const T
   }
 }
 
-template <typename TM, typename SI, typename SO>
-static int matvec_go(int N, const void* inv, const void* x, void* y, int nrhs, int acc, const int* midx,
-                     cudaStream_t st) {
-  typedef typename Store<TM>::R R;
-  const unsigned gx = (unsigned)((N + kMvRows - 1) / kMvRows);
-  constexpr int kRB = sizeof(R) == 8 ? 2 : 4;
-  const size_t most = (size_t)smem_optin_bytes() - 2048;
-  const bool one = nrhs == 1 || midx || (size_t)kRB * N * sizeof(cx<R>) > most;
-  const size_t sm = (size_t)(one ? 1 : kRB) * N * sizeof(cx<R>);
-  if (sm > most) return -1;  // above 8192 rows, which no hierarchy has
-#define WMG_MV(B)                                                                                                 \
-  {                                                                                                               \
-    auto kern = dense_matvec_kernel<TM, SI, SO, B>;                                                               \
-    if (sm > 40 * 1024) allow_big_smem(kern);                                                                     \
-    launch_chain(kern, dim3(gx, (unsigned)((nrhs + B - 1) / B)), kMvThreads, sm, st, N, (const TM*)inv, (const SI*)x, \
-                 (SO*)y, nrhs, acc, midx);                                                                        \
-  }
-  if (one)
-    WMG_MV(1)
-  else
-    WMG_MV(kRB)
-#undef WMG_MV
+template <typename TM, typename SI, typename SO, int ROWS, bool PIECES>
+static int matvec_rows(int N, const void* inv, const void* x, void* y, int nrhs, int acc, const int* midx, cudaStream_t st) {
+  auto kern = dense_matvec_kernel<TM, SI, SO, ROWS, PIECES>;
+  const dim3 grid((unsigned)((N + ROWS - 1) / ROWS), (unsigned)nrhs);
+  const size_t sm = (size_t)(PIECES ? kMvPiece : N) * sizeof(cx<typename Store<TM>::R>);
+  if (sm > (size_t)smem_optin_bytes() - 2048) return -1;  // FP32 above 28,000 rows, which no hierarchy has
+  if (sm > 40 * 1024) allow_big_smem(kern);
+  static std::atomic<unsigned long long> held{0};
+  const ChainOff crowded(N >= 1024 && !chain_fits((long)grid.x * grid.y, ctas_held(held, kern, 64 * ROWS, sm), sm_count()));
+  launch_chain(kern, grid, 64 * ROWS, sm, st, N, (const TM*)inv, (const SI*)x, (SO*)y, acc, midx);
   return launched() ? 0 : -1;
 }
 
-// Right-hand sides up to which the row form runs: it reads the matrix once per
-// four, the tiled product once (N = 1536: 12 right-hand sides 36 us against 53,
-// 24 61 against 60; N = 768, 48: 33 against 27).
-constexpr int kMvMost = 16;
+template <typename TM, typename SI, typename SO>
+static int matvec_go(int N, const void* inv, const void* x, void* y, int nrhs, int acc, const int* midx,
+                     cudaStream_t st) {
+  if constexpr (sizeof(TM) == 16) {
+    const bool two = matvec_rows_per_cta(N, nrhs, sm_count()) == 2;
+    if (N > 2 * kMvPiece)
+      return two ? matvec_rows<TM, SI, SO, 2, true>(N, inv, x, y, nrhs, acc, midx, st)
+                 : matvec_rows<TM, SI, SO, 4, true>(N, inv, x, y, nrhs, acc, midx, st);
+    if (two) return matvec_rows<TM, SI, SO, 2, false>(N, inv, x, y, nrhs, acc, midx, st);
+  }
+  return matvec_rows<TM, SI, SO, 4, false>(N, inv, x, y, nrhs, acc, midx, st);
+}
 
 int launch_dense_matvec(int pm, int pin, int pout, int N, const void* inv, const void* x, void* y, int nrhs, int acc,
                         cudaStream_t st, void* scratch, const int* midx) {
-  if (nrhs <= kMvMost || !scratch || midx) {
+  if (nrhs <= matvec_most(pm, N) || !scratch || midx) {
     int rc = -1;
     if (pm == 0 && pin == 0 && pout == 0)
       rc = matvec_go<double2, double2, double2>(N, inv, x, y, nrhs, acc, midx, st);
@@ -1269,11 +1277,11 @@ int launch_dense_matvec(int pm, int pin, int pout, int N, const void* inv, const
     const dim3 g(tiles, KS);
     unsigned* tickets = (unsigned*)((char*)scratch + (size_t)8 * 64 * N * 16);
     if (pm == 0 && pin == 0 && pout == 0)
-      launch_chain(dense_matmul_kernel<double2, double2, double2>, g, kMmThreads, 0, st, N, (const double2*)inv, (const double2*)x, (double2*)y, nrhs, acc, kper, (cx<double>*)scratch, tickets);
+      matmul_go(dense_matmul_kernel<double2, double2, double2>, g, st, N, (const double2*)inv, (const double2*)x, (double2*)y, nrhs, acc, kper, (cx<double>*)scratch, tickets);
     else if (pm == 1 && pin == 0 && pout == 0)
-      launch_chain(dense_matmul_kernel<float2, double2, double2>, g, kMmThreads, 0, st, N, (const float2*)inv, (const double2*)x, (double2*)y, nrhs, acc, kper, (cx<float>*)scratch, tickets);
+      matmul_go(dense_matmul_kernel<float2, double2, double2>, g, st, N, (const float2*)inv, (const double2*)x, (double2*)y, nrhs, acc, kper, (cx<float>*)scratch, tickets);
     else if (pm == 1 && pin == 1 && pout == 1)
-      launch_chain(dense_matmul_kernel<float2, float2, float2>, g, kMmThreads, 0, st, N, (const float2*)inv, (const float2*)x, (float2*)y, nrhs, acc, kper, (cx<float>*)scratch, tickets);
+      matmul_go(dense_matmul_kernel<float2, float2, float2>, g, st, N, (const float2*)inv, (const float2*)x, (float2*)y, nrhs, acc, kper, (cx<float>*)scratch, tickets);
     else
       return -1;
     return launched() ? 0 : -1;

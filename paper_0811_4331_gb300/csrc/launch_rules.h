@@ -98,6 +98,20 @@ inline CoarseShape coarse_shape(size_t elem, long n, long V, int nrhs, int sms) 
   return {1, rb, lb, pitch(lb)};
 }
 
+// ------------------------------------------------------------------ coarsest product
+// Right-hand sides up to which the row form runs: it reads the matrix once for
+// each, the tiled product once for all.  FP32, N = 1536: 16 right-hand sides 37 us
+// against 50, 24 53 against 56; N = 4096 (a matrix as large as the L2): 12 279
+// against 321, 16 368 against 338; N = 8192: 12 1053 against 1259, 16 1393 against
+// 1327.  FP64: both are bound by arithmetic, of which the tiled product does 64
+// right-hand sides' in any case (N = 1536, 24: 420 against 1320).
+inline int matvec_most(int prec, long N) { return prec == 0 || N <= 3584 ? 16 : 12; }
+// FP64: rows of a CTA, four or two, by the fuller of the SMs (N = 2048: 512 CTAs of four are four on some SMs).
+inline int matvec_rows_per_cta(long N, int nrhs, int sms) {
+  auto time = [&](long rows) { return ((N + rows - 1) / rows * nrhs + sms - 1) / sms * rows; };
+  return 100 * time(2) < 97 * time(4) ? 2 : 4;
+}
+
 // ------------------------------------------------------------------ fine stencil
 // Threads an SM is to hold, one thread per site, for elements of `elem` bytes,
 // i.e. the register budget (65,536 / threads).  Measured (us per launch; "-":
@@ -145,6 +159,27 @@ inline int dot_tiles(long tiles, long lanes, int per_sm, int sms, int elem) {
   int best = most;
   while (100 * time(best) > 103 * least) --best;
   return best;
+}
+
+// ------------------------------------------------------------------ Gram-Schmidt dots
+// Blocks per lane (a chunk of eight vectors and a right-hand side) for `tiles`
+// tiles of 256 elements: at least four tiles each, one block per SM; where few
+// lanes leave the SMs with less than four FP32 or two FP64 blocks, more of them as
+// long as each has eight (FP32) or sixteen tiles.  25 M elements, up to 8 vectors,
+// one right-hand side: FP32 701 -> 272 us, FP64 1877 -> 1350 (four blocks on
+// 393,216 elements: 43 us instead of 29).  FP32 blocks stay whole waves of four
+// per SM (1.5 M elements, 40 vectors, five lanes: 88 us with a block per SM and lane, 77).
+inline int multidot_grid(long tiles, int lanes, int elem, int sms, int most) {
+  const long few = (tiles + 3) / 4, each = elem == 16 ? 16 : 8;
+  const long want = elem == 16 ? 2 : 4, cap = sms * ((want + lanes - 1) / lanes);
+  long b = few;
+  if (b > sms) {
+    b = tiles / each > sms ? tiles / each : sms;
+    b = b > cap ? cap : b;
+    if (elem != 16 && lanes > 4) b = 4L * sms * (lanes / 4) / lanes;
+  }
+  b = b > most ? most : b;
+  return (int)(b < 1 ? 1 : b);
 }
 
 // ------------------------------------------------------------------ chained launches

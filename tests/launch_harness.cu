@@ -35,3 +35,17 @@ extern "C" int t_coarse_mma(const void* C, void* packed, const void* in, void* o
 }
 extern "C" size_t t_mma_pack_bytes(int n, int V) { return mma_pack_bytes(n, V); }
 extern "C" size_t t_mma_scratch_bytes(int n, int V, int R) { return coarse_mma_scratch_bytes(n, V, R); }
+
+// Coarsest product y = inv x, row form or tiled (scratch zeroed).
+extern "C" int t_matvec(int pm, int pin, int pout, int N, const void* inv, const void* x, void* y, int nrhs, int acc,
+                        void* scratch) {
+  return launch_dense_matvec(pm, pin, pout, N, inv, x, y, nrhs, acc, nullptr, scratch, nullptr);
+}
+extern "C" size_t t_matvec_scratch_bytes(int N) { return dense_matvec_scratch_bytes(N); }
+
+// Overlaps <W_j|w> of right-hand side r at result[(r kmax + j) 2]; W holds a multiple of eight vectors.
+extern "C" int t_multidot(int prec, size_t n, int nrhs, int k, int kmax, const void* W, const void* w, double* partials,
+                          unsigned* tickets, double* result) {
+  const RedArgs red = {partials, tickets, result, 0};
+  return launch_multidot(prec, n, nrhs, k, kmax, W, n * nrhs, w, red, nullptr);
+}

@@ -19,7 +19,7 @@ def load():
                         "-fPIC", "-I", build.CSRC, os.path.join(_here, "launch_harness.cu"), "-o", out, "-L", pkg,
                         "-lwilsonmg", "-Xlinker", "-rpath=" + pkg], check=True)
         _loaded = ctypes.CDLL(out)
-        for f in ("t_mma_pack_bytes", "t_mma_scratch_bytes"):
+        for f in ("t_mma_pack_bytes", "t_mma_scratch_bytes", "t_matvec_scratch_bytes"):
             getattr(_loaded, f).restype = ctypes.c_size_t
     return _loaded
 

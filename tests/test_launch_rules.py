@@ -78,3 +78,14 @@ def test_dot_tiles_fill_their_waves(tmp_path):
         assert 1 <= k <= 32 and time(k) <= 1.031 * min(time(q) for q in range(1, 33)), (tiles, lanes, per_sm)
     src = open(os.path.join(CSRC, "wilson.cu")).read()
     assert "dot_tiles(grid.x, nrhs / NR, wilson_threads<S, NR, true>() / NT" in src
+
+
+def test_coarsest_product_and_dots(tmp_path):
+    """Row form: two rows per FP64 CTA where four leave an SM with a fifth more; FP32 above 3,584 rows goes to the tiled
+    product with 13.  Overlaps: more blocks only on long vectors and few lanes, at most the partial buffer's."""
+    rows = _run(tmp_path, "\n".join("printf(\"%%d\\n\", %s);" % e for e in (
+        "matvec_rows_per_cta(2048, 1, 152)", "matvec_rows_per_cta(1216, 1, 152)", "matvec_most(1, 3072)",
+        "matvec_most(1, 4096)", "matvec_most(0, 8192)", "multidot_grid(384, 1, 8, 152, 1216)",
+        "multidot_grid(98304, 1, 8, 152, 1216)", "multidot_grid(98304, 1, 16, 152, 1216)",
+        "multidot_grid(98304, 5, 8, 152, 1216)", "multidot_grid(98304, 12, 8, 152, 1216)", "multidot_grid(1, 1, 8, 152, 1216)")))
+    assert [r[0] for r in rows] == [2, 4, 16, 12, 16, 96, 608, 304, 121, 152, 1]
