@@ -226,18 +226,17 @@ __device__ __forceinline__ R warp_sum16(const R (&v)[16]) {
   return d + __shfl_xor_sync(0xffffffffu, d, 1);
 }
 
-// Blocks per chunk and right-hand side: at least 4 elements per thread, at most one block per SM.
-static int multidot_blocks(size_t n) {
-  const size_t b = (n + 4 * kVecThreads - 1) / (4 * kVecThreads);
-  const size_t cap = (size_t)sm_count() < (size_t)kMaxVecBlocks ? (size_t)sm_count() : (size_t)kMaxVecBlocks;
-  return (int)(b > cap ? cap : (b < 1 ? 1 : b));
+// Blocks per chunk and right-hand side (launch_rules.h).
+static int multidot_blocks(size_t n, int lanes, int elem) {
+  return multidot_grid((long)((n + kVecThreads - 1) / kVecThreads), lanes, elem, sm_count(), kMaxVecBlocks);
 }
 
 // On small lattices the reduction of the 16 sums was most of the time (a tree of
 // FP64 additions per value in the last block): 8^3 x 16 (98,304 elements), up to
-// 8 vectors, 18.5 -> 6.8 us.
-template <typename S>
-__global__ void __launch_bounds__(kVecThreads)
+// 8 vectors, 18.5 -> 6.8 us.  On large ones FP32 is bound by the loads in flight:
+// PAIRS takes two elements per load (16 bytes).
+template <typename S, bool PAIRS>
+__global__ void __launch_bounds__(kVecThreads, 4)  // a launch of two blocks per SM then fits beside the one before it
     multidot_kernel(size_t n, int k, int kmax, const S* W, size_t jstride, const S* w, RedArgs ra,
                     const double* pre, const double* post, int cstride) {
   chain_begin();
@@ -255,14 +254,29 @@ __global__ void __launch_bounds__(kVecThreads)
   cx<R> acc[kChunk];
 #pragma unroll
   for (int q = 0; q < kChunk; ++q) acc[q] = zero<R>();
+  const size_t i0 = (size_t)blockIdx.x * kVecThreads + threadIdx.x, step = (size_t)gridDim.x * kVecThreads;
+  if constexpr (PAIRS) {
+    for (size_t i = i0; i < n / 2; i += step) {
+      const float4 x = __ldg(reinterpret_cast<const float4*>(wr) + i);
+      float4 v[kChunk];
+#pragma unroll
+      for (int q = 0; q < kChunk; ++q) v[q] = __ldg(reinterpret_cast<const float4*>(Wc + (size_t)q * jstride) + i);
+#pragma unroll
+      for (int q = 0; q < kChunk; ++q) {
+        acc[q] = cfma_conj(mk<R>(v[q].x, v[q].y), mk<R>(x.x, x.y), acc[q]);
+        acc[q] = cfma_conj(mk<R>(v[q].z, v[q].w), mk<R>(x.z, x.w), acc[q]);
+      }
+    }
+  } else {
 #pragma unroll 2
-  for (size_t i = (size_t)blockIdx.x * kVecThreads + threadIdx.x; i < n; i += (size_t)gridDim.x * kVecThreads) {
-    const cx<R> x = ldc<R>(wr, i);
-    cx<R> v[kChunk];
+    for (size_t i = i0; i < n; i += step) {
+      const cx<R> x = ldc<R>(wr, i);
+      cx<R> v[kChunk];
 #pragma unroll
-    for (int q = 0; q < kChunk; ++q) v[q] = ldc<R>(Wc + (size_t)q * jstride, i);
+      for (int q = 0; q < kChunk; ++q) v[q] = ldc<R>(Wc + (size_t)q * jstride, i);
 #pragma unroll
-    for (int q = 0; q < kChunk; ++q) acc[q] = cfma_conj(v[q], x, acc[q]);
+      for (int q = 0; q < kChunk; ++q) acc[q] = cfma_conj(v[q], x, acc[q]);
+    }
   }
   R red[NV];
 #pragma unroll
@@ -307,15 +321,20 @@ int launch_multidot(int prec, size_t n, int nrhs, int k, int kmax, const void* W
                     RedArgs red, cudaStream_t st, const double* pre, const double* post, int cstride) {
   if (k <= 0) return 0;
   if (kmax % kChunk) return -1;
-  dim3 grid(multidot_blocks(n), (k + kChunk - 1) / kChunk, nrhs);
+  const int chunks = (k + kChunk - 1) / kChunk;
+  dim3 grid(multidot_blocks(n, chunks * nrhs, prec == 0 ? 16 : 8), chunks, nrhs);
   switch (prec) {
     case 0:
-      launch_chain(multidot_kernel<double2>, grid, kVecThreads, 0, st, n, k, kmax, (const double2*)W, jstride,
+      launch_chain(multidot_kernel<double2, false>, grid, kVecThreads, 0, st, n, k, kmax, (const double2*)W, jstride,
                    (const double2*)w, red, pre, post, cstride);
       break;
     case 1:
-      launch_chain(multidot_kernel<float2>, grid, kVecThreads, 0, st, n, k, kmax, (const float2*)W, jstride,
-                   (const float2*)w, red, pre, post, cstride);
+      if (n % 2 == 0 && jstride % 2 == 0 && (((uintptr_t)W | (uintptr_t)w) & 15u) == 0)
+        launch_chain(multidot_kernel<float2, true>, grid, kVecThreads, 0, st, n, k, kmax, (const float2*)W, jstride,
+                     (const float2*)w, red, pre, post, cstride);
+      else
+        launch_chain(multidot_kernel<float2, false>, grid, kVecThreads, 0, st, n, k, kmax, (const float2*)W, jstride,
+                     (const float2*)w, red, pre, post, cstride);
       break;
     default: return -1;
   }
