@@ -59,11 +59,10 @@ __device__ __forceinline__ void ld_sites(const S* p, cx<R> (&v)[BV]) {
 // CTA (deterministic).  With one right-hand side the operator's bytes bound it
 // (85 MB on 512 sites, n = 48, FP32), with several in FP64 the FP64 pipe.
 // The operator is read once per RB right-hand sides.
-// 512 sites, n = 48, FP32, one right-hand side: 33 -> 20.7 us (18 with
-// chained launches), 12: 243 -> 77; 32 sites, FP64, one (n = 40): 16.5 -> 12.5
-// us, 12 (n = 48): 97 -> 66.
+// 512 sites, n = 48, FP32, one right-hand side: 33 -> 15.9 us, 12: 243 -> 64; 32
+// sites, FP64, n = 48, 12: 97 -> 62 us; 36 sites, FP64, n = 64, 24: 287 -> 224.
 template <typename S, int BV, int IR, int RB, int LB>
-__global__ void 
+__global__ void
     __launch_bounds__(256, sizeof(S) == 8 && BV == 2 && IR * RB == 2 ? 3 : 0)  // two registers above three per SM
     coarse_apply_kernel(const CoarseArgs<S> A, int pitch, int nrhs) {
   chain_begin();
@@ -1134,11 +1133,15 @@ __global__ void __launch_bounds__(kMmThreads)
 // complex FP64) and one ticket per 16-row tile.
 // A launch of about two CTAs per SM, bound by arithmetic: an SM with three would set its time (N = 2048, FP64, 24
 // right-hand sides: 2344 us, crowded 3588).
-template <typename K, typename... A>
-static void matmul_go(K kern, dim3 grid, cudaStream_t st, A... args) {
+template <typename TM, typename SI, typename SO>
+static int matmul_go(dim3 grid, cudaStream_t st, int N, const void* inv, const void* x, void* y, int nrhs, int acc, int kper,
+                     void* scratch, unsigned* tickets) {
+  auto kern = dense_matmul_kernel<TM, SI, SO>;
   static const int per_sm = ctas_per_sm(kern, kMmThreads, 0);
   const ChainOff crowded(!chain_fits((long)grid.x * grid.y, per_sm, sm_count()));
-  launch_chain(kern, grid, kMmThreads, 0, st, args...);
+  launch_chain(kern, grid, kMmThreads, 0, st, N, (const TM*)inv, (const SI*)x, (SO*)y, nrhs, acc, kper,
+               (cx<typename Store<TM>::R>*)scratch, tickets);
+  return launched() ? 0 : -1;
 }
 
 size_t dense_matvec_scratch_bytes(int N) {
@@ -1277,14 +1280,11 @@ int launch_dense_matvec(int pm, int pin, int pout, int N, const void* inv, const
     const dim3 g(tiles, KS);
     unsigned* tickets = (unsigned*)((char*)scratch + (size_t)8 * 64 * N * 16);
     if (pm == 0 && pin == 0 && pout == 0)
-      matmul_go(dense_matmul_kernel<double2, double2, double2>, g, st, N, (const double2*)inv, (const double2*)x, (double2*)y, nrhs, acc, kper, (cx<double>*)scratch, tickets);
-    else if (pm == 1 && pin == 0 && pout == 0)
-      matmul_go(dense_matmul_kernel<float2, double2, double2>, g, st, N, (const float2*)inv, (const double2*)x, (double2*)y, nrhs, acc, kper, (cx<float>*)scratch, tickets);
-    else if (pm == 1 && pin == 1 && pout == 1)
-      matmul_go(dense_matmul_kernel<float2, float2, float2>, g, st, N, (const float2*)inv, (const float2*)x, (float2*)y, nrhs, acc, kper, (cx<float>*)scratch, tickets);
-    else
-      return -1;
-    return launched() ? 0 : -1;
+      return matmul_go<double2, double2, double2>(g, st, N, inv, x, y, nrhs, acc, kper, scratch, tickets);
+    if (pm == 1 && pin == 0 && pout == 0)
+      return matmul_go<float2, double2, double2>(g, st, N, inv, x, y, nrhs, acc, kper, scratch, tickets);
+    if (pm == 1 && pin == 1 && pout == 1)
+      return matmul_go<float2, float2, float2>(g, st, N, inv, x, y, nrhs, acc, kper, scratch, tickets);
   }
   return -1;
 }
