@@ -67,15 +67,22 @@ inline int sm_count() {
 // steps in BF16 (six launches): 49 -> 41 us; 360 launches of a Gauss-Jordan
 // inverse: 6.7 -> 5.9 ms.  Everything after chain_begin() sees its
 // predecessors' memory; a kernel without it is launched with <<<>>>.
-// Not inside a graph capture: a graph's edges cost little by themselves, and
-// there the early blocks took places unevenly (twelve-source solve 309 -> 333
-// ms); nor where a launch of one wave depends on an even placement (the fused
-// setup step, 13.4 -> 14.6 ms of setup).
+// An early grid takes the places that its predecessor leaves, so where CTAs run
+// long and few, some SMs get more of them than others: chain_fits (launch_rules.h)
+// keeps FP64 launches and the coarsest product from that, ChainOff the cases below.
+// Off in the library's own captures (a graph's edges cost little by themselves,
+// and the twelve-source solve took 333 ms with early starts, 309 without), among
+// the solves of mg_solve_many (four on 8^3 x 16: 17.1 and 16.7 ms), for FP64
+// transfers inside a cycle, and for one-wave launches of the fused setup step (14.6
+// and 13.4 ms of setup).  On in a caller's capture (20 FP16 stencils on 8^3 x 16: 51
+// us, 59 without; two BF16 MR steps gain 4 %, the tile transfers lose 2 %) and in
+// solves on a caller's threads (mg_solve_masses on two threads: one right-hand side
+// 8.2 ms, 8.6 without; eight 20.6 and 20.3).
 __device__ __forceinline__ void chain_begin() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
-inline thread_local bool tl_chain_off = false;  // set while this thread captures a graph or solves beside others
+inline thread_local bool tl_chain_off = false;  // set by ChainOff
 // While alive (and `off`), this thread's launch_chain launches wait for their predecessor's end.
 struct ChainOff {
   const bool prev = tl_chain_off;
